@@ -452,7 +452,7 @@ __device__ __forceinline__ void moments_post(const Par& p, const R (&f)[19], R& 
 
 // ---------------------------------------------------------------------------
 // Plane / unit-cube volume (piecewise cubic in the plane constant alpha for a
-// normal with sorted components m1 <= m2 <= m3, m1+m2+m3 = 1) and its slope.
+// normal with sorted components m1 <= m2 <= m3, m1+m2+m3 = 1).
 // ---------------------------------------------------------------------------
 template <class R>
 __device__ __forceinline__ R cube_vol_half(R a, R m1, R m2, R m3) {
@@ -478,30 +478,6 @@ __device__ __forceinline__ R cube_vol(R a, R m1, R m2, R m3) {
   if (a > R(0.5)) return R(1) - cube_vol_half(R(1) - a, m1, m2, m3);
   return cube_vol_half(a, m1, m2, m3);
 }
-template <class R>
-__device__ __forceinline__ R cube_area_half(R a, R m1, R m2, R m3) {
-  if (a <= R(0)) return R(0);
-  if (a <= m1) return a * a / (R(2) * m1 * m2 * m3);
-  R base = R(6) * a - R(3) * m1;
-  R den = R(6) * m2 * m3;
-  if (a <= m2) return base / den;
-  R s = a - m2;
-  R m12 = m1 + m2;
-  if (m3 >= m12) {
-    if (a <= m12) return (base - R(3) * s * s / m1) / den;
-    return R(1) / m3;
-  }
-  if (a <= m3) return (base - R(3) * s * s / m1) / den;
-  R r = a - m3;
-  return (base - R(3) * s * s / m1 - R(3) * r * r / m1) / den;
-}
-template <class R>
-__device__ __forceinline__ R cube_area(R a, R m1, R m2, R m3) {
-  if (a >= R(1)) return R(0);
-  if (a > R(0.5)) return cube_area_half(R(1) - a, m1, m2, m3);
-  return cube_area_half(a, m1, m2, m3);
-}
-
 // Inverse of cube_vol_half by region, for the float forms: with the sorted
 // normal (m1 <= m2 <= m3, sum 1) the volume is alpha^3 / (6 m1 m2 m3) on
 // [0, m1] (a cube root), a quadratic on [m1, m2] (a square root), linear on
@@ -565,16 +541,102 @@ __host__ __device__ __forceinline__ R plic_alpha_regions(R tv, R m1, R m2, R m3)
   return al;
 }
 
+// a / b in float for a correction that only has to be right to a few digits
+__host__ __device__ __forceinline__ float fast_quot(float a, float b) {
+#ifdef __CUDA_ARCH__
+  return __fdividef(a, b);
+#else
+  return a / b;
+#endif
+}
+
+// The same inverse in FP64, for the FP64 form.  GB300 issues two FP64
+// operations per cycle and SM, and a bracketing search of 20 steps with its
+// divisions spent over a thousand of them per open cell and set the time of
+// the FP64 geometry kernel (283 us alone for 57 k interface cells of a
+// 256x128x128 splash; that lattice's step 1048 -> 695 us with this inverse,
+// a 128^3 wave's 681 -> 619 us).  Here the region of the root is chosen by
+// the volumes at its ends as above, float arithmetic gives the root to its
+// own resolution (1e-7 relative), and each polishing step takes the
+// volume's residual in FP64, without divisions (multiplied through by the
+// region's denominators), and its slope and quotient in float: the error
+// shrinks by 1e-7 or more a step, so two steps reach FP64 rounding and a third
+// is kept on the cubic ranges.
+__host__ __device__ __forceinline__ double plic_alpha_polished(double tv, double m1, double m2, double m3) {
+  const double m12 = m1 + m2, den = 6.0 * (m2 * m3), tden = tv * den, m11 = m1 * m1;
+  if (m1 > 0.0 && tden <= m11) {  // alpha^3 = 6 m1 m2 m3 tv
+    const double c = tden * m1;
+    double al = (double)cbrtf((float)c);
+#pragma unroll
+    for (int it = 0; it < 2; ++it) {
+      const float af = (float)al;
+      al -= (double)fast_quot((float)(al * al * al - c), 3.0f * af * af);
+    }
+    return al;
+  }
+  const double v2 = 3.0 * m2 * (m2 - m1) + m11;  // V(m2) den
+  if (m2 > 0.0 && tden <= v2) {
+    const double t = tden * (1.0 / 3.0) - m11 * (1.0 / 12.0);
+    if (!(t > 0.0)) return 0.5 * m1;
+    double r = (double)sqrtf((float)t);
+#pragma unroll
+    for (int it = 0; it < 2; ++it) r -= (double)fast_quot((float)(r * r - t), 2.0f * (float)r);
+    return 0.5 * m1 + r;
+  }
+  double lo = m2, hi = m12;
+  bool four = false;  // the range [m3, 1/2] of a cube with m3 < m1 + m2
+  const double t3 = tden * m1;
+  if (m3 >= m12) {
+    if (tv * m3 >= 0.5 * m12) return m3 * tv + 0.5 * m12;
+  } else {
+    const double s = m3 - m2;
+    four = t3 > m1 * (3.0 * m3 * (m3 - m1) + m11) - s * s * s;
+    lo = four ? m3 : m2;
+    hi = four ? 0.5 : m3;
+  }
+  // cubic ranges (m1 > 0): m1 (3 a^2 - 3 a m1 + m1^2) - (a - m2)^3 [- (a - m3)^3] = 6 m1 m2 m3 tv
+  const float f1 = (float)m1, f2 = (float)m2, f3 = (float)m3, flo = (float)lo, fhi = (float)hi, ft = (float)t3;
+  auto slope = [&](float a) {
+    const float s = a - f2, r = four ? a - f3 : 0.0f;
+    return f1 * (6.0f * a - 3.0f * f1) - 3.0f * (s * s + r * r);
+  };
+  float a = 0.5f * (flo + fhi);
+#pragma unroll 1
+  for (int it = 0; it < 5; ++it) {
+    const float s = a - f2, r = four ? a - f3 : 0.0f, dv = slope(a);
+    if (!(dv > 0.0f)) break;
+    const float v = f1 * (3.0f * a * (a - f1) + f1 * f1) - (s * s * s + r * r * r);
+    const float nx = a - fast_quot(v - ft, dv);
+    a = nx < flo ? flo : (nx > fhi ? fhi : nx);
+  }
+  double al = (double)a;
+#pragma unroll
+  for (int it = 0; it < 3; ++it) {
+    const double s = al - m2, r = four ? al - m3 : 0.0;
+    const double v = m1 * (3.0 * al * (al - m1) + m11) - (s * s * s + r * r * r);
+    const float dv = slope((float)al);
+    if (!(dv > 0.0f)) break;
+    const double nx = al - (double)fast_quot((float)(v - t3), dv);
+    al = nx < lo ? lo : (nx > hi ? hi : nx);
+  }
+  return al;
+}
+
 // Signed offset d (from the cell centre along the unit normal n, liquid on
 // the side n.(x - x_c) <= d) of the plane cutting volume fraction ph.  The
 // fill is kept in [1e-9, 1 - 1e-9] first: at an empty or full corner the
 // inverse volume grows like a cube root and would turn rounding of ph into
-// visible plane shifts.  Bracketing bisection, then Newton on the convex half.
+// visible plane shifts.
 template <class R>
 __device__ R plic_offset(R nx_, R ny_, R nz_, R ph) {
   R a0 = fabs(nx_), a1 = fabs(ny_), a2 = fabs(nz_);
   R L1 = a0 + a1 + a2;
-  a0 /= L1; a1 /= L1; a2 /= L1;
+  if constexpr (sizeof(R) == 8) {  // (one FP64 division for three)
+    const R il = R(1) / L1;
+    a0 *= il; a1 *= il; a2 *= il;
+  } else {
+    a0 /= L1; a1 /= L1; a2 /= L1;
+  }
   // sort ascending
   R t;
   if (a0 > a1) { t = a0; a0 = a1; a1 = t; }
@@ -591,23 +653,7 @@ __device__ R plic_offset(R nx_, R ny_, R nz_, R ph) {
     if (upper) al = R(1) - al;
     return L1 * (al - R(0.5));
   }
-  R lo = R(0), hi = R(0.5);
-#pragma unroll 1
-  for (int it = 0; it < 20; ++it) {  // bracket to 2^-21
-    R mid = R(0.5) * (lo + hi);
-    if (cube_vol_half(mid, a0, a1, a2) < tv) lo = mid; else hi = mid;
-  }
-  // Newton from the right end of the bracket (convex, increasing: monotone),
-  // kept inside the bracket
-  R al = hi;
-  constexpr int newton = sizeof(R) == 8 ? 6 : 3;
-#pragma unroll 1
-  for (int it = 0; it < newton; ++it) {
-    R ar = cube_area_half(al, a0, a1, a2);
-    if (!(ar > R(0))) break;
-    R nx2 = al - (cube_vol_half(al, a0, a1, a2) - tv) / ar;
-    al = nx2 < lo ? lo : (nx2 > hi ? hi : nx2);
-  }
+  R al = (R)plic_alpha_polished(tv, a0, a1, a2);
   if (upper) al = R(1) - al;
   return L1 * (al - R(0.5));
 }
@@ -951,8 +997,8 @@ __device__ __forceinline__ void geometry(const Par& p, const uint8_t* __restrict
       const R il = rsqrtf(v0 * v0 + v1 * v1 + v2 * v2);
       n[0] = v0 * il; n[1] = v1 * il; n[2] = v2 * il;
     } else {
-      R len = sqrt(v0 * v0 + v1 * v1 + v2 * v2);
-      n[0] = v0 / len; n[1] = v1 / len; n[2] = v2 / len;
+      const R il = R(1) / sqrt(v0 * v0 + v1 * v1 + v2 * v2);
+      n[0] = v0 * il; n[1] = v1 * il; n[2] = v2 * il;
     }
     R nabs = fabs(a == 0 ? n[0] : (a == 1 ? n[1] : n[2]));
     d = nabs * (H[4] - R(3.5));
@@ -976,8 +1022,8 @@ __device__ __forceinline__ void geometry(const Par& p, const uint8_t* __restrict
       const R il = rsqrtf(nn);
       n[0] *= il; n[1] *= il; n[2] *= il;
     } else {
-      R len = sqrt(nn);
-      n[0] /= len; n[1] /= len; n[2] /= len;
+      const R il = R(1) / sqrt(nn);
+      n[0] *= il; n[1] *= il; n[2] *= il;
     }
     d = plic_offset<R>(n[0], n[1], n[2], phic);
   }
