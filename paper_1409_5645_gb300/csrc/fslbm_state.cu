@@ -7,9 +7,10 @@ namespace fsl {
 // Populations from the caller (pre-collision f, or f^eq(rho,u) + noise) ->
 // collide -> stored f~(t); m = phi rho, phi = m/rho on interface cells.
 template <int P>
-__global__ void k_init_pre(Par p, View<P> v, const double* __restrict__ fin, const double* __restrict__ phi,
-                           const double* __restrict__ rho_in, const double* __restrict__ u_in,
-                           const double* __restrict__ noise, double* __restrict__ keep_f0) {
+__global__ void __launch_bounds__(128, P == P64 ? 4 : 6)
+    k_init_pre(Par p, View<P> v, const double* __restrict__ fin, const double* __restrict__ phi,
+               const double* __restrict__ rho_in, const double* __restrict__ u_in, const double* __restrict__ noise,
+               double* __restrict__ keep_f0) {
   using R = typename Form<P>::R;
   const size_t N = (size_t)p.N;
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < p.N;
@@ -26,23 +27,41 @@ __global__ void k_init_pre(Par p, View<P> v, const double* __restrict__ fin, con
 #pragma unroll
       for (int q = 0; q < 19; ++q) fd[q] = fin[(size_t)q * N + i];
     } else {
-      // equilibrium at (rho, u), u^eq = u (Eq. eqEven / eqOdd)
-      double r = rho_in[i], u0 = u_in[3 * i], u1 = u_in[3 * i + 1], u2 = u_in[3 * i + 2];
-      double r0 = p.compressible ? r : 1.0;
-      double usq = u0 * u0 + u1 * u1 + u2 * u2;
-      fd[0] = eplus<double, 0>(p, r, r0, u0, u1, u2, usq);
-#define FSL_EQ(q) fd[q] = eplus<double, q>(p, r, r0, u0, u1, u2, usq) + eminus<double, q>(r0, u0, u1, u2);
-      FSL_EQ(1) FSL_EQ(2) FSL_EQ(3) FSL_EQ(4) FSL_EQ(5) FSL_EQ(6) FSL_EQ(7) FSL_EQ(8) FSL_EQ(9)
-      FSL_EQ(10) FSL_EQ(11) FSL_EQ(12) FSL_EQ(13) FSL_EQ(14) FSL_EQ(15) FSL_EQ(16) FSL_EQ(17) FSL_EQ(18)
-#undef FSL_EQ
+      // equilibrium at (rho, u), u^eq = u (Eq. eqEven / eqOdd): both
+      // directions of a link share e^+ and take e^- with opposite signs (the
+      // FP64 pipe bounds this kernel, so each is formed once; the roundings are
+      // those of the expressions of eplus and eminus; 512x256x256, FP32 form:
+      // 2.73 -> 1.67 ms)
+      const double r = rho_in[i];
+      const double u[3] = {u_in[3 * i], u_in[3 * i + 1], u_in[3 * i + 2]};
+      const double r0 = p.compressible ? r : 1.0, nl = p.linear_eq ? 0.0 : 1.0;
+      const double usq = fma(u[2], u[2], fma(u[0], u[0], u[1] * u[1]));
+      fd[0] = fma(wq<double>(0), r, -(((wq<double>(0) * 1.5) * r0 * nl) * usq));
+      const double wr1 = wq<double>(1) * r, wr7 = wq<double>(7) * r;
+      const double k1 = (wq<double>(1) * 1.5) * r0 * nl, k7 = (wq<double>(7) * 1.5) * r0 * nl;
+      const double o1 = (3.0 * wq<double>(1)) * r0, o7 = (3.0 * wq<double>(7)) * r0;
+#pragma unroll
+      for (int q = 1; q < 19; q += 2) {
+        double cu = 0.0;
+        if (cx(q)) cu = cx(q) > 0 ? u[0] : -u[0];
+        if (cy(q)) cu = cy(q) > 0 ? cu + u[1] : cu - u[1];
+        if (cz(q)) cu = cz(q) > 0 ? cu + u[2] : cu - u[2];
+        const double ep = fma(q <= 6 ? k1 : k7, fma(3.0 * cu, cu, -usq), q <= 6 ? wr1 : wr7);
+        fd[q] = fma(q <= 6 ? o1 : o7, cu, ep);
+        fd[q + 1] = fma(-(q <= 6 ? o1 : o7), cu, ep);
+      }
       if (noise) {
 #pragma unroll
         for (int q = 0; q < 19; ++q) fd[q] += noise[(size_t)q * N + i];
       }
     }
     double rs = 0.0;
+    if (k == IFC || fin || noise) {
 #pragma unroll
-    for (int q = 0; q < 19; ++q) rs += fd[q];
+      for (int q = 0; q < 19; ++q) rs += fd[q];
+    } else {
+      rs = rho_in[i];  // (the equilibrium's sum; a liquid cell's m is read by nothing)
+    }
     if (keep_f0) {
 #pragma unroll
       for (int q = 0; q < 19; ++q) keep_f0[(size_t)q * N + i] = fd[q];
@@ -88,57 +107,209 @@ __global__ void k_init_post(Par p, View<P> v, const double* __restrict__ fpost, 
 }
 
 // NEARB bit (a link ends in a wall or past a face) and invariant checks.
+__device__ __forceinline__ void prepare_cell(const Par& p, uint8_t* flags, int* err, long long i, int x, int y, int z) {
+  const uint8_t k = flags[i] & KIND;
+  if (k != LIQ && k != IFC && k != GAS && k != WALL) {
+    atomicOr(err, ERRB_STATE);
+    return;
+  }
+  bool nearb = false, nearw = false, gas = false;
+#pragma unroll
+  for (int q = 1; q < 19; ++q) {
+    long long j = nbr(p, x, y, z, cx(q), cy(q), cz(q));
+    uint8_t kj = kind_at(flags, j);
+    nearb |= (kj == WALL);
+    nearw |= (j >= 0 && kj == WALL);
+    gas |= (kj == GAS);
+  }
+  if (k == LIQ && gas) atomicOr(err, ERRB_STATE);
+  flags[i] = (uint8_t)(k | (nearb ? NEARB : 0) | (nearw ? NEARW : 0));
+}
 __global__ void k_prepare_flags(Par p, uint8_t* flags, int* err) {
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < p.N;
        i += (long long)gridDim.x * blockDim.x) {
-    uint8_t k = flags[i] & KIND;
-    if (k != LIQ && k != IFC && k != GAS && k != WALL) { atomicOr(err, ERRB_STATE); continue; }
     int x, y, z;
     coords(p, i, x, y, z);
-    bool nearb = false, nearw = false, gas = false;
-#pragma unroll
-    for (int q = 1; q < 19; ++q) {
-      long long j = nbr(p, x, y, z, cx(q), cy(q), cz(q));
-      uint8_t kj = kind_at(flags, j);
-      nearb |= (kj == WALL);
-      nearw |= (j >= 0 && kj == WALL);
-      gas |= (kj == GAS);
+    prepare_cell(p, flags, err, i, x, y, z);
+  }
+}
+// The same with 16 cells of a row per thread (nx a multiple of 16): the kinds
+// are one-hot, so the OR of the neighbours' bytes holds their kinds; nine
+// 16-byte loads and ten single bytes instead of 18 bytes a cell (512x256x256:
+// 953 -> 96 us).  Cells on the y and z faces, and a row's
+// first and last group on a periodic x axis, take the cell path.  The bits written beside
+// the kinds are masked from every load, so cells may be rewritten while their
+// neighbours read them.
+__global__ void __launch_bounds__(256) k_prepare_flags16(Par p, uint8_t* flags, int* err) {
+  const long long total = p.N >> 4;
+  const long long sy = p.nx, sz = (long long)p.nx * p.ny;
+  for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < total;
+       t += (long long)gridDim.x * blockDim.x) {
+    const long long i = t << 4;
+    int x, y, z;
+    coords(p, i, x, y, z);
+    const bool xlo = x == 0, xhi = x + 16 == p.nx;
+    if (((xlo || xhi) && p.px) || y == 0 || y == p.ny - 1 || z == 0 || z == p.nz - 1) {
+      for (int k = 0; k < 16; ++k) prepare_cell(p, flags, err, i + k, x + k, y, z);
+      continue;
     }
-    if (k == LIQ && gas) atomicOr(err, ERRB_STATE);
-    flags[i] = (uint8_t)(k | (nearb ? NEARB : 0) | (nearw ? NEARW : 0));
+    unsigned near[4] = {0u, 0u, 0u, 0u}, own[4] = {0u, 0u, 0u, 0u};
+#pragma unroll
+    for (int dz = -1; dz <= 1; ++dz)
+#pragma unroll
+      for (int dy = -1; dy <= 1; ++dy) {
+        const uint8_t* row = flags + (i + dy * sy + dz * sz);
+        const uint4 w4 = *reinterpret_cast<const uint4*>(row);
+        const unsigned w[4] = {w4.x, w4.y, w4.z, w4.w};
+        const bool centre = dy == 0 && dz == 0;
+        if (!centre) {
+#pragma unroll
+          for (int k = 0; k < 4; ++k) near[k] |= w[k];
+        }
+        if (dy == 0 || dz == 0) {  // the links along x too
+          const unsigned before = xlo ? 0u : row[-1], after = xhi ? 0u : row[16];
+#pragma unroll
+          for (int k = 0; k < 4; ++k) {
+            near[k] |= (w[k] << 8) | (k ? w[k - 1] >> 24 : before);
+            near[k] |= (w[k] >> 8) | ((k < 3 ? w[k + 1] : after) << 24);
+          }
+        }
+        if (centre) {
+#pragma unroll
+          for (int k = 0; k < 4; ++k) own[k] = w[k] & 0x0f0f0f0fu;
+        }
+      }
+    bool bad = false;
+    uint4 out;
+    unsigned* o = &out.x;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const unsigned one = 0x01010101u, b0 = own[k] & one, b1 = (own[k] >> 1) & one, b2 = (own[k] >> 2) & one,
+                     b3 = (own[k] >> 3) & one;
+      bad = bad || b0 + b1 + b2 + b3 != one;                  // each byte one kind (no carry: at most 4)
+      bad = bad || (b0 & ((near[k] >> 2) & one)) != 0u;       // a liquid cell next to gas
+      const unsigned wall = (near[k] >> 3) & one;
+      o[k] = own[k] | (wall * (unsigned)(NEARB | NEARW));
+    }
+    if (xlo) o[0] |= NEARB;  // (beyond a non-periodic face: a wall)
+    if (xhi) o[3] |= (unsigned)NEARB << 24;
+    if (bad) atomicOr(err, ERRB_STATE);
+    *reinterpret_cast<uint4*>(flags + i) = out;
   }
 }
 
-template <int P>
-__global__ void k_fields(Par p, View<P> v, unsigned mask, uint8_t* oflags, double* of, double* om, double* ophi,
-                         double* orho, double* ou) {
+// one 8- or 16-byte store of VEC doubles
+template <int VEC>
+struct VecT;
+template <>
+struct VecT<1> {
+  using T = double;
+  static __device__ __forceinline__ T of(const double* a) { return a[0]; }
+};
+template <>
+struct VecT<2> {
+  using T = double2;
+  static __device__ __forceinline__ T of(const double* a) { return make_double2(a[0], a[1]); }
+};
+
+// The fields of VEC x-adjacent cells per thread (VEC = 2 where N is even, so
+// that every plane's pairs are 16-byte aligned).  The velocities, three per
+// cell, go through shared memory so that a warp's stores are whole sectors.
+// The 512x256x256 read-back (every field, FP32 form) writes 6.7 GB: 2.54 ms
+// with a cell per thread and the velocities stored 24 bytes apart, 1.83 ms so
+// (0.54 of the copy bandwidth).
+template <int P, int VEC>
+__global__ void __launch_bounds__(128) k_fields(Par p, View<P> v, unsigned mask, uint8_t* oflags, double* of,
+                                                double* om, double* ophi, double* orho, double* ou) {
+  using S = typename Form<P>::S;
   using R = typename Form<P>::R;
+  constexpr bool SH = Form<P>::SH;
+  struct alignas(8 * VEC) Vec { double a[VEC]; };
+  struct alignas(sizeof(S) * VEC) SVec { S a[VEC]; };
+  __shared__ double su[128 * 3 * VEC];
   const size_t N = (size_t)p.N;
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < p.N;
-       i += (long long)gridDim.x * blockDim.x) {
-    uint8_t k = v.flags[i] & KIND;
-    bool fl = is_fluid(k);
-    constexpr bool SH = Form<P>::SH;
-    R f[19];
+  const long long n = p.N / VEC;
+  for (long long b0 = (long long)blockIdx.x * 128; b0 < n; b0 += (long long)gridDim.x * 128) {
+    const long long t = b0 + threadIdx.x;
+    const bool in = t < n;
+    const long long i = t * VEC;
+    double ux[VEC][3];
+    if (in) {
+      uint8_t k[VEC];
+      bool any = false, fl[VEC];
 #pragma unroll
-    for (int q = 0; q < 19; ++q) f[q] = fl ? ldq<P>(v.fin, (size_t)q * N + i, q) : R(0);
-    R rho = R(0), ux = R(0), uy = R(0), uz = R(0);
-    if (fl) moments_post<R, SH>(p, f, rho, ux, uy, uz);
-    const double rhof = fl ? rho_full<SH>(rho) : 0.0;
-    if (oflags) oflags[i] = k;
-    if (of) {
+      for (int c = 0; c < VEC; ++c) {
+        k[c] = v.flags[i + c] & KIND;
+        fl[c] = is_fluid(k[c]);
+        any = any || fl[c];
+      }
+      any = any && (of || om || orho || ou);  // (kinds and fill levels alone read no population)
+      R f[VEC][19];
+      if (any) {
 #pragma unroll
-      for (int q = 0; q < 19; ++q) of[(size_t)q * N + i] = fl ? ldq_full<P>(v.fin, (size_t)q * N + i, q) : 0.0;
+        for (int q = 0; q < 19; ++q) {
+          const SVec w = *reinterpret_cast<const SVec*>(v.fin + (size_t)q * N + i);
+#pragma unroll
+          for (int c = 0; c < VEC; ++c) {
+            R val;
+            if constexpr (P == P16) val = __half2float(w.a[c]);
+            else val = w.a[c];
+            f[c][q] = fl[c] ? val : R(0);
+          }
+        }
+      } else {
+#pragma unroll
+        for (int q = 0; q < 19; ++q)
+#pragma unroll
+          for (int c = 0; c < VEC; ++c) f[c][q] = R(0);
+      }
+      if (of) {
+#pragma unroll
+        for (int q = 0; q < 19; ++q) {
+          Vec w;
+#pragma unroll
+          for (int c = 0; c < VEC; ++c) {
+            w.a[c] = (double)f[c][q];
+            if constexpr (SH) {
+              if (any) w.a[c] = fl[c] ? w.a[c] + wq<double>(q) : 0.0;
+            }
+          }
+          __stcs(reinterpret_cast<typename VecT<VEC>::T*>(of + (size_t)q * N + i), VecT<VEC>::of(w.a));
+        }
+      }
+      Vec wm, wp, wr;
+#pragma unroll
+      for (int c = 0; c < VEC; ++c) {
+        R rho = R(0), vx = R(0), vy = R(0), vz = R(0);
+        if (fl[c]) moments_post<R, SH>(p, f[c], rho, vx, vy, vz);
+        const double rhof = fl[c] ? rho_full<SH>(rho) : 0.0;
+        if (oflags) oflags[i + c] = k[c];
+        wm.a[c] = !om ? 0.0 : (k[c] == IFC ? v.m[i + c] : (k[c] == LIQ ? rhof : 0.0));
+        double ph = 0.0;
+        if (k[c] == LIQ) ph = 1.0;
+        else if (ophi && (k[c] == IFC || (k[c] == GAS && p.freeze))) ph = (double)v.phin[i + c];
+        wp.a[c] = ph;
+        wr.a[c] = rhof;
+        ux[c][0] = (double)vx; ux[c][1] = (double)vy; ux[c][2] = (double)vz;
+      }
+      using T = typename VecT<VEC>::T;
+      if (om) __stcs(reinterpret_cast<T*>(om + i), VecT<VEC>::of(wm.a));
+      if (ophi) __stcs(reinterpret_cast<T*>(ophi + i), VecT<VEC>::of(wp.a));
+      if (orho) __stcs(reinterpret_cast<T*>(orho + i), VecT<VEC>::of(wr.a));
     }
-    if (om) om[i] = k == IFC ? v.m[i] : (k == LIQ ? rhof : 0.0);
-    if (ophi) {
-      double ph = 0.0;
-      if (k == LIQ) ph = 1.0;
-      else if (k == IFC || (k == GAS && p.freeze)) ph = (double)v.phin[i];
-      ophi[i] = ph;
+    if (ou) {
+      if (in) {
+#pragma unroll
+        for (int c = 0; c < VEC; ++c)
+#pragma unroll
+          for (int a = 0; a < 3; ++a) su[(threadIdx.x * VEC + c) * 3 + a] = ux[c][a];
+      }
+      __syncthreads();
+      const long long left = (n - b0 < 128 ? n - b0 : 128) * VEC * 3;
+      double* dst = ou + b0 * VEC * 3;
+      for (int e = threadIdx.x; e < left; e += 128) __stcs(dst + e, su[e]);
+      __syncthreads();
     }
-    if (orho) orho[i] = rhof;
-    if (ou) { ou[3 * i] = (double)ux; ou[3 * i + 1] = (double)uy; ou[3 * i + 2] = (double)uz; }
   }
 }
 
@@ -196,7 +367,10 @@ int launch_init_post(const Par& p, const View<P>& v, const double* f, const doub
   return (int)cudaGetLastError();
 }
 int launch_prepare_flags(const Par& p, uint8_t* flags, int* err, cudaStream_t st) {
-  k_prepare_flags<<<grid_for(p.N, 256), 256, 0, st>>>(p, flags, err);
+  if ((p.nx & 15) == 0)
+    k_prepare_flags16<<<grid_for(p.N / 16, 256), 256, 0, st>>>(p, flags, err);
+  else
+    k_prepare_flags<<<grid_for(p.N, 256), 256, 0, st>>>(p, flags, err);
   return (int)cudaGetLastError();
 }
 template <int P>
@@ -205,8 +379,13 @@ int launch_fields(const Par& p, const View<P>& v, unsigned mask, void* const* ou
   int k = 0;
   for (int b = 0; b < 6; ++b)
     if (mask & (1u << b)) ptr[b] = out[k++];
-  k_fields<P><<<grid_for(p.N, 128), 128, 0, st>>>(p, v, mask, (uint8_t*)ptr[0], (double*)ptr[1], (double*)ptr[2],
-                                                   (double*)ptr[3], (double*)ptr[4], (double*)ptr[5]);
+  // (the callers' buffers need not be 16-byte aligned)
+  bool pairs = (p.N & 1) == 0;
+  for (int b = 1; b < 6; ++b) pairs = pairs && ((uintptr_t)ptr[b] & 15) == 0;
+  auto kernel = pairs ? k_fields<P, 2> : k_fields<P, 1>;
+  kernel<<<grid_for(pairs ? p.N / 2 : p.N, 128), 128, 0, st>>>(p, v, mask, (uint8_t*)ptr[0], (double*)ptr[1],
+                                                               (double*)ptr[2], (double*)ptr[3], (double*)ptr[4],
+                                                               (double*)ptr[5]);
   return (int)cudaGetLastError();
 }
 template <int P>
