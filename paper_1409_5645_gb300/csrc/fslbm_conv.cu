@@ -67,15 +67,12 @@ __device__ __forceinline__ double rho_out(const Par& p, const View<P>& v, long l
   return rho_full<Form<P>::SH>(r);
 }
 
-// one warp per fill cell, lane q (1..18) takes link q
+// fill cell k by a warp, lane q (1..18) takes link q
 template <int P>
-__device__ __forceinline__ void do_fill(const Par& p, const View<P>& v) {
+__device__ __forceinline__ void fill_cell(const Par& p, const View<P>& v, int k) {
   const int lane = threadIdx.x & 31;
-  const int gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int nw = (gridDim.x * blockDim.x) >> 5;
-  const int nf = min(load_count(&v.cnt[1]), v.cap);
   const int q = (lane >= 1 && lane < 19) ? lane : 0;
-  for (int k = gw; k < nf; k += nw) {
+  {
     const long long i = FSL_CK(p, v.flist[k], p.N);
     int x, y, z;
     coords(p, i, x, y, z);
@@ -92,28 +89,16 @@ __device__ __forceinline__ void do_fill(const Par& p, const View<P>& v) {
     push(won, v.nglist, &v.cnt[3], v.cap, (int)j, v.err);
   }
 }
-template <int P>
-__device__ __forceinline__ void do_empty(const Par& p, const View<P>& v);
-template <int P>
-__global__ void __launch_bounds__(256) k_fill_empty(Par p, View<P> v) {
-  pdl_begin();
-  do_fill<P>(p, v);
-  do_empty<P>(p, v);
-}
-
-// one warp per new cell: lane l (1..18) reads neighbour l's populations; the
+// new cell k by a warp: lane l (1..18) reads neighbour l's populations; the
 // means are summed in neighbour order; lane q builds and collides population q
 template <int P>
-__device__ __forceinline__ void do_newg(const Par& p, const View<P>& v) {
+__device__ __forceinline__ void newg_cell(const Par& p, const View<P>& v, int k) {
   using R = typename Form<P>::R;
   const unsigned FULL = 0xffffffffu;
   const size_t N = (size_t)p.N;
   const int lane = threadIdx.x & 31;
-  const int gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int nw = (gridDim.x * blockDim.x) >> 5;
-  const int nn = min(load_count(&v.cnt[3]), v.cap);
   const int q = lane < 19 ? lane : 0;
-  for (int k = gw; k < nn; k += nw) {
+  {
     const long long j = FSL_CK(p, v.nglist[k], p.N);
     int x, y, z;
     coords(p, j, x, y, z);
@@ -140,7 +125,13 @@ __device__ __forceinline__ void do_newg(const Par& p, const View<P>& v) {
       if (ul) { rs += a; s0 += b0; s1 += b1; s2 += b2; ++c; }
     }
     // (rbar is rho - 1 in the shifted forms: the mean of rho - 1)
-    const R rbar = rs / R(c), u0 = s0 / R(c), u1 = s1 / R(c), u2 = s2 / R(c);
+    R rbar, u0, u1, u2;
+    if constexpr (P == P64) {  // (one FP64 division for four: they bound the FP64 form's stage)
+      const R ic = R(1) / R(c);
+      rbar = rs * ic; u0 = s0 * ic; u1 = s1 * ic; u2 = s2 * ic;
+    } else {
+      rbar = rs / R(c); u0 = s0 / R(c); u1 = s1 / R(c); u2 = s2 / R(c);
+    }
     const R r0 = p.compressible ? rho_full_r<Form<P>::SH>(rbar) : R(1);
     const R usq = u0 * u0 + u1 * u1 + u2 * u2;
     const R wq_ = q == 0 ? R(1) / R(3) : (q <= 6 ? R(1) / R(18) : R(1) / R(36));
@@ -158,10 +149,15 @@ __device__ __forceinline__ void do_newg(const Par& p, const View<P>& v) {
       jz += __shfl_xor_sync(FULL, jz, o);
     }
     const R rc = p.compressible ? rho_full_r<Form<P>::SH>(rho) : R(1);
-    const R Ux = jx / rc, Uy = jy / rc, Uz = jz / rc;
+    R Ux = jx, Uy = jy, Uz = jz;
+    if (p.compressible) {
+      Ux = jx / rc;
+      Uy = jy / rc;
+      Uz = jz / rc;
+    }
     const R gx = R(p.g[0]), gy = R(p.g[1]), gz = R(p.g[2]);
     const R vx_ = Ux + R(0.5) * gx, vy_ = Uy + R(0.5) * gy, vz_ = Uz + R(0.5) * gz;
-    const R ilm = R(1) / R(p.lam_m);
+    const R ilm = P == P64 ? R(p.inv_lam_m) : R(1) / R(p.lam_m);
     const R ex = Ux - gx * ilm, ey = Uy - gy * ilm, ez = Uz - gz * ilm;
     const R usq2 = vx_ * vx_ + vy_ * vy_ + vz_ * vz_;
     const R fb = __shfl_sync(FULL, f, inv(q));
@@ -176,17 +172,14 @@ __device__ __forceinline__ void do_newg(const Par& p, const View<P>& v) {
   }
 }
 
-// one warp per empty cell still marked, lane q (1..18) takes link q
+// empty cell k (still marked: only its own warp clears that) by a warp, lane q
+// (1..18) takes link q
 template <int P>
-__device__ __forceinline__ void do_empty(const Par& p, const View<P>& v) {
+__device__ __forceinline__ void empty_cell(const Par& p, const View<P>& v, int k) {
   const int lane = threadIdx.x & 31;
-  const int gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int nw = (gridDim.x * blockDim.x) >> 5;
-  const int ne = min(load_count(&v.cnt[2]), v.cap);
   const int q = (lane >= 1 && lane < 19) ? lane : 0;
-  for (int k = gw; k < ne; k += nw) {
+  {
     const long long i = FSL_CK(p, v.elist[k], p.N);
-    if (!(v.mark[i] & MK_EMPTY)) continue;  // warp-uniform
     int x, y, z;
     coords(p, i, x, y, z);
     long long j = -1;
@@ -201,7 +194,7 @@ __device__ __forceinline__ void do_empty(const Par& p, const View<P>& v) {
     // an emptied cell next to a filled one stays interface
     if (__any_sync(0xffffffffu, (mj & MK_FILL) != 0)) {
       if (lane == 0) clear_u8(v.mark, i, MK_EMPTY);
-      continue;  // (warp-uniform)
+      return;  // (warp-uniform)
     }
     bool won = false;
     if (kj == LIQ) {
@@ -212,12 +205,31 @@ __device__ __forceinline__ void do_empty(const Par& p, const View<P>& v) {
   }
 }
 
+// the first stage: a warp per fill or empty cell
+template <int P>
+__device__ __forceinline__ void do_fill_empty(const Par& p, const View<P>& v) {
+  const int nf = min(load_count(&v.cnt[1]), v.cap), ne = min(load_count(&v.cnt[2]), v.cap);
+  const int nw = (gridDim.x * blockDim.x) >> 5;
+  for (int k = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; k < nf + ne; k += nw) {
+    if (k < nf) fill_cell<P>(p, v, k);
+    else empty_cell<P>(p, v, k - nf);
+  }
+}
+template <int P>
+__global__ void __launch_bounds__(256) k_fill_empty(Par p, View<P> v) {
+  pdl_begin();
+  do_fill_empty<P>(p, v);
+}
+
 // liquid cells turned interface next to an emptied cell: m = rho, phi = m/rho
+// (by the grid's last threads first: its first warps take the other items of
+// the stage)
 template <int P>
 __device__ __forceinline__ void do_newl(const Par& p, const View<P>& v) {
   using R = typename Form<P>::R;
   int nl = min(load_count(&v.cnt[4]), v.cap);
-  for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < nl; k += gridDim.x * blockDim.x) {
+  const int nt = gridDim.x * blockDim.x;
+  for (int k = nt - 1 - (int)(blockIdx.x * blockDim.x + threadIdx.x); k < nl; k += nt) {
     long long j = FSL_CK(p, v.nllist[k], p.N);
     const double r = rho_out<P>(p, v, j);
     v.m[j] = r;
@@ -255,20 +267,18 @@ __device__ __forceinline__ double split_weight(const double (&n)[3], int ax, int
   return filled ? (d > 0.0 ? d : 0.0) : (d < 0.0 ? -d : 0.0);
 }
 
-// one warp per fill / empty cell: lane q (1..18) tests neighbour q as a
-// receiver; lane 0 computes the share (rho summed in q order, as a thread would)
+// fill or empty cell k (of nf fills, then the empties) by a warp: lane q (1..18)
+// tests neighbour q as a receiver; lane 0 computes the share (rho summed in q
+// order, as a thread would)
 template <int P>
-__device__ __forceinline__ void do_share(const Par& p, const View<P>& v) {
+__device__ __forceinline__ void share_cell(const Par& p, const View<P>& v, int k, int nf) {
   const unsigned FULL = 0xffffffffu;
   const int lane = threadIdx.x & 31;
-  const int gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int nw = (gridDim.x * blockDim.x) >> 5;
-  const int nf = min(load_count(&v.cnt[1]), v.cap), ne = min(load_count(&v.cnt[2]), v.cap);
   const int q = (lane >= 1 && lane < 19) ? lane : 0;
-  for (int k = gw; k < nf + ne; k += nw) {
+  {
     const bool isF = k < nf;
     const long long i = FSL_CK(p, isF ? v.flist[k] : v.elist[k - nf], p.N);
-    if (!isF && !(v.mark[i] & MK_EMPTY)) continue;  // warp-uniform
+    if (!isF && !(v.mark[i] & MK_EMPTY)) return;  // warp-uniform
     int x, y, z;
     coords(p, i, x, y, z);
     // lane 0: the cell's density and mass, loaded beside the neighbour tests
@@ -321,13 +331,23 @@ __device__ __forceinline__ void do_share(const Par& p, const View<P>& v) {
 
 // new cells from gas, new cells from liquid and the excess shares are
 // independent once the first stage has claimed the new cells and settled the
-// empty list
+// empty list: their items follow one another over the grid's warps, so that a
+// warp has one of them (not one of each) until every warp has one
+template <int P>
+__device__ __forceinline__ void do_new_share(const Par& p, const View<P>& v) {
+  const int nf = min(load_count(&v.cnt[1]), v.cap), ne = min(load_count(&v.cnt[2]), v.cap);
+  const int nn = min(load_count(&v.cnt[3]), v.cap);
+  const int nw = (gridDim.x * blockDim.x) >> 5;
+  for (int k = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; k < nn + nf + ne; k += nw) {
+    if (k < nn) newg_cell<P>(p, v, k);
+    else share_cell<P>(p, v, k - nn, nf);
+  }
+  do_newl<P>(p, v);
+}
 template <int P>
 __global__ void __launch_bounds__(256) k_new_share(Par p, View<P> v) {
   pdl_begin();
-  do_newg<P>(p, v);
-  do_newl<P>(p, v);
-  do_share<P>(p, v);
+  do_new_share<P>(p, v);
 }
 
 // one thread per receiver (the lists are long late in a run): gathers the
@@ -346,19 +366,36 @@ __device__ __forceinline__ void do_recv(const Par& p, const View<P>& v) {
     // neighbours' marks and shares
     const double m0 = v.m[yj];
     const double rho = p.excess_split ? 1.0 : rho_out<P>(p, v, yj);
-    double acc = 0.0;
+    // the neighbours' marks, then the converting ones' shares, each as loads
+    // in flight together (a load, a test and a dependent load per neighbour in
+    // turn took 13 us of a 128x64x64 splash's 41 us conversions)
+    unsigned conv = 0u, wsp = 0u;
+    int jq[19];
 #pragma unroll
     for (int q = 1; q < 19; ++q) {
       const long long j = in1 ? yj + (cx(q) + sy * cy(q) + sz * cz(q)) : nbr(p, x, y, z, cx(q), cy(q), cz(q));
-      if (j < 0) continue;
-      const uint8_t mk = v.mark[j];
-      if (mk & (MK_FILL | MK_EMPTY)) {
-        if (mk & MK_WSPLIT) {  // the link from j to this receiver is -c_q
+      jq[q] = (int)j;
+      const uint8_t mk = j < 0 ? (uint8_t)0 : v.mark[j];
+      if (mk & (MK_FILL | MK_EMPTY)) conv |= 1u << q;
+      if (mk & MK_WSPLIT) wsp |= 1u << q;
+    }
+    double acc = 0.0, sh[19];
+#pragma unroll
+    for (int q = 1; q < 19; ++q) sh[q] = (conv & (1u << q)) ? v.share[jq[q]] : 0.0;
+    if (!(conv & wsp)) {
+#pragma unroll
+      for (int q = 1; q < 19; ++q)
+        if (conv & (1u << q)) acc += sh[q];
+    } else {
+#pragma unroll
+      for (int q = 1; q < 19; ++q) {
+        if (!(conv & (1u << q))) continue;
+        if (wsp & (1u << q)) {  // the link from j to this receiver is -c_q
           double n[3];
-          fill_normal<P>(p, v, j, n);
-          acc += v.share[j] * split_weight(n, -cx(q), -cy(q), -cz(q), (mk & MK_FILL) != 0);
+          fill_normal<P>(p, v, jq[q], n);
+          acc += sh[q] * split_weight(n, -cx(q), -cy(q), -cz(q), (v.mark[jq[q]] & MK_FILL) != 0);
         } else {
-          acc += v.share[j];
+          acc += sh[q];
         }
       }
     }
@@ -468,30 +505,39 @@ __device__ __forceinline__ void grid_sync(unsigned* ctr, unsigned target, int* e
 }
 
 // the four conversion stages in one launch, separated by grid barriers; the
-// step's two-level mass reduction rides along in the first two stages (the
-// same chunks and order as the stand-alone reduction), with the lost ledger
-// read before any excess of this step reaches it
+// step's two-level mass reduction (the same chunks and order as the
+// stand-alone pair of launches) is carried by the grid's last blocks, the
+// last of them to finish its chunk adding up the chunks: it reads the lost
+// ledger before its block arrives at the first barrier, so before any excess
+// of this step reaches it.  A step without a fill or an empty cell ends there
+// (alone, with warm caches: a film's step 17.2 -> 6.8 us; with conversions, the
+// items of a stage spread over the warps and the receivers' loads together,
+// a 128x64x64 splash's 46.8 -> 35.0 us)
 template <int P>
 __global__ void __launch_bounds__(256) k_convert(Par p, View<P> v, MassReduce mr) {
   pdl_begin();
   unsigned* ctr = (unsigned*)&v.cnt[10];
   const unsigned nb = gridDim.x;
-  double lost0 = 0.0;
-  if (mr.nb > 0 && blockIdx.x == 0 && threadIdx.x == 0) lost0 = *mr.add;
-  if ((int)blockIdx.x < mr.nb) {
-    const double t = block_chunk_sum(mr.in, mr.n, mr.chunk, blockIdx.x);
-    if (threadIdx.x == 0) mr.tmp[blockIdx.x] = t;
+  const int chunk = (int)blockIdx.x - ((int)gridDim.x - mr.nb);
+  if (chunk >= 0) {
+    __shared__ bool last;
+    const double t = block_chunk_sum(mr.in, mr.n, mr.chunk, chunk);
+    if (threadIdx.x == 0) {
+      mr.tmp[chunk] = t;
+      __threadfence();
+      last = atomicAdd(&v.cnt[11], 1) == mr.nb - 1;
+      __threadfence();
+    }
+    __syncthreads();
+    if (last) {
+      const double m = block_chunk_sum<true>(mr.tmp, mr.nb, mr.nb, 0);
+      if (threadIdx.x == 0) *mr.out = m + *mr.add;
+    }
   }
-  do_fill<P>(p, v);
-  do_empty<P>(p, v);
+  if (load_count(&v.cnt[1]) + load_count(&v.cnt[2]) == 0) return;  // (settled before this kernel)
+  do_fill_empty<P>(p, v);
   grid_sync(ctr, nb, v.err);
-  if (mr.nb > 0 && blockIdx.x == 0) {
-    const double t = block_chunk_sum(mr.tmp, mr.nb, mr.nb, 0);
-    if (threadIdx.x == 0) *mr.out = t + lost0;
-  }
-  do_newg<P>(p, v);
-  do_newl<P>(p, v);
-  do_share<P>(p, v);
+  do_new_share<P>(p, v);
   grid_sync(ctr, 2 * nb, v.err);
   do_recv<P>(p, v);
   grid_sync(ctr, 3 * nb, v.err);

@@ -255,7 +255,8 @@ struct View {
   int* nllist;  // new from liquid
   int* rlist;   // excess receivers
   int* cnt;     // [0] ilist front [6] ilist back [1] flist [2] elist [3] ng [4] nl [5] rl [7] emptied;
-                // [8] all conversions since set; [9] fluid segments; [10] grid barrier of k_convert
+                // [8] all conversions since set; [9] fluid segments; [10] grid barrier of k_convert;
+                // [11] blocks of it that have summed their chunk of the mass
   int cap;
   double* share;
   R* geo;            // interface geometry per list entry: [5][cap] n0, n1, n2, d, kappa (n = 0: none)
@@ -1032,13 +1033,14 @@ __device__ __forceinline__ void geometry(const Par& p, const uint8_t* __restrict
 // Fixed-order sum of chunk b of in[0, n) by the calling block of 256 threads:
 // strided per-thread sums, warp shuffles, the eight warp sums in a fixed
 // tree.  Every thread of the block must call it; the result is on thread 0.
-__device__ __forceinline__ double block_chunk_sum(const double* __restrict__ in, long long n, long long chunk,
-                                                  long long b) {
+// CG: the values were written by other blocks of the running kernel (read at L2).
+template <bool CG = false>
+__device__ __forceinline__ double block_chunk_sum(const double* in, long long n, long long chunk, long long b) {
   __shared__ double red[8];
   const long long lo = b * chunk;
   const long long hi = lo + chunk < n ? lo + chunk : n;
   double s = 0.0;
-  for (long long k = lo + threadIdx.x; k < hi; k += blockDim.x) s += in[k];
+  for (long long k = lo + threadIdx.x; k < hi; k += blockDim.x) s += CG ? __ldcg(in + k) : in[k];
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
   if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;

@@ -40,7 +40,7 @@ inline int launch_k(void (*kernel)(KArgs...), unsigned grid, unsigned block, siz
 int launch_segments(const Par& p, const uint8_t* flags, int* seglist, int* segcount, int* ilist, int* cnt, int cap,
                     int* err, cudaStream_t st);
 
-// zero the per-step counters cnt[0..7] and cnt[9] (one small kernel, so that
+// zero the per-step counters cnt[0..7] and cnt[9..11] (one small kernel, so that
 // the whole step is a chain of kernels)
 int launch_reset(int* cnt, cudaStream_t st);
 

@@ -176,7 +176,7 @@ int launch_segments(const Par& p, const uint8_t* flags, int* seglist, int* segco
 
 __global__ void k_reset(int* cnt) {
   pdl_begin();
-  if (threadIdx.x < 11 && threadIdx.x != 8) cnt[threadIdx.x] = 0;
+  if (threadIdx.x < 12 && threadIdx.x != 8) cnt[threadIdx.x] = 0;
 }
 
 int launch_reset(int* cnt, cudaStream_t st) { return launch_k(k_reset, 1, 32, 0, st, cnt); }
