@@ -173,7 +173,9 @@ extern "C" int fslbm_adjoint_forward(fslbm_t* h, int nsteps, int K, int objectiv
                    A->ck_flags + s * N))
       return adj_fail(h, FSLBM_ERR_CUDA, "checkpoint copy");
     int n = nsteps - s * K < K ? nsteps - s * K : K;
+    h->fp64_chain = 1;
     int rc = fslbm_step(h, n);
+    h->fp64_chain = 0;
     if (rc) return rc;
   }
   cudaEventRecord(e1, h->st);

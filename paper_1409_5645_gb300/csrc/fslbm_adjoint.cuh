@@ -952,7 +952,10 @@ int adj_backward(fslbm* h) {
       if (save_state(h, (char*)A->seg_f + k * A->fbytes, A->seg_m + k * N, (char*)A->seg_phi + k * A->rbytes,
                      A->seg_flags + k * N))
         return 1;
-      if (k < n && fslbm_step(h, 1)) return 1;
+      h->fp64_chain = 1;
+      const int rc = k < n ? fslbm_step(h, 1) : 0;
+      h->fp64_chain = 0;
+      if (rc) return 1;
     }
     cudaEventRecord(e0, st);
     for (int k = n - 1; k >= 0; --k) {

@@ -6,6 +6,7 @@
 //   (2 kernels) -> 7 conversion kernels (dynamic interface only)
 // and swaps the A/B population and fill-level buffers.
 #include <cuda_runtime.h>
+#include <math.h>
 #include <stdio.h>
 #include <vector>
 #include <stdlib.h>
@@ -174,6 +175,22 @@ extern "C" int fslbm_create_ex(const fslbm_params* prm, fslbm_t** out) {
   p.elvira = q.elvira;
   p.adj32 = q.adjoint_fp32 && q.precision != FSLBM_F64;
   p.umax2 = q.u_max * q.u_max;
+  {
+    // the FP64 form's collision in fixed point: |lambda| < 2 holds for every
+    // tau > 1/2; the forces must leave the operands in range
+    bool ok = !p.compressible && !p.linear_eq;
+    for (int a = 0; a < 3; ++a) {
+      const double gl = p.g[a] * p.inv_lam_m;
+      ok = ok && fabs(p.g[a]) < 1.0 / 32.0 && fabs(gl) < 1.0 / 8.0;
+      p.fx_hg[a] = ok ? llround(p.g[a] * 0x1p59) : 0;
+      p.fx_gl[a] = ok ? llround(gl * 0x1p60) : 0;
+    }
+    ok = ok && p.lam_p > -2.0 && p.lam_p < 0.0 && p.lam_m > -2.0 && p.lam_m < 0.0;
+    p.fx_lp = ok ? llround(p.lam_p * 0x1p62) : 0;
+    p.fx_lm = ok ? llround(p.lam_m * 0x1p62) : 0;
+    p.fx_um2 = p.umax2 > 0.0 && p.umax2 < 4.0 ? llround(p.umax2 * 0x1p60) : 0x7fffffffffffffffLL;
+    p.fix_ok = ok;
+  }
 
   const size_t Nn = (size_t)N, N4 = (Nn + 3) & ~(size_t)3;
   h->cap = (int)N;
@@ -496,8 +513,10 @@ static int mark_event(fslbm* h, int k) {
 template <int P>
 static int step_t(fslbm* h) {
   View<P> v = make_view<P>(h);
+  Par par = h->par;
+  if (h->fp64_chain) par.fix_ok = 0;
   if (launch_reset(h->cnt, h->st)) return 1;
-  if (launch_step_kernels<P>(h->par, v, h->st, h->bulk_blocks, h->iface_blocks, h->seglist, h->cnt + 9,
+  if (launch_step_kernels<P>(par, v, h->st, h->bulk_blocks, h->iface_blocks, h->seglist, h->cnt + 9,
                              h->timing ? h : nullptr, h->bulk_mode, h->tmap ? &h->tmap[h->cur] : nullptr,
                              (h->forked && h->overlap) ? &h->fork : nullptr))
     return 1;

@@ -159,6 +159,17 @@ struct Par {
   int elvira;              // 1: ELVIRA normal where the height columns are open
   int adj32;               // 1: the adjoint's reverse step in FP32 (FP32/FP16 lattices)
   double umax2;            // stability guard: |u|^2 above it is an error (0: off)
+  // FP64 form: the collision's constants in fixed point (fslbm_fixed.cuh);
+  // fix_ok: they are in its range and the default equilibria are in use.  The
+  // steps of a differentiation run with fix_ok = 0: a gradient can be the
+  // small remainder of terms that cancel over the window (an 8x4x64 film's
+  // dJ/dnu and dJ/dphi0 after 200 steps moved by 1e-7 with the last bits of
+  // the state), so there the FP64 operations stay those they have always been.
+  int fix_ok;
+  long long fx_lp, fx_lm;  // lambda_+-, units of 2^-62
+  long long fx_hg[3];      // g / 2, units of 2^-60
+  long long fx_gl[3];      // g / lambda_-
+  long long fx_um2;        // u_max^2 (the largest value: off)
 #ifdef FSLBM_CHECKED
   int* err;                // the handle's error word (bounds-checked build)
 #endif

@@ -56,6 +56,7 @@ struct fslbm {
   fsl::Fork fork;     // the side stream of the interface kernels and its two events
   int forked;         // fork holds a stream and events
   int overlap;        // 1: the interface kernels run on the side stream beside the bulk kernel
+  int fp64_chain;     // the steps of a differentiation: the FP64 form without the fixed-point collision (Par::fix_ok)
 };
 
 

@@ -81,6 +81,10 @@ template <int P>
 int launch_bulk_pairs(const Par& p, const View<P>& v, cudaStream_t st, int bulk_blocks, const int* seglist,
                       const int* segcount, bool shared);
 
+// FP64 bulk kernel, collision in fixed point (fslbm_bulk64.cu)
+int launch_bulk_fixed(const Par& p, const View<P64>& v, cudaStream_t st, int bulk_blocks, const int* seglist,
+                      const int* segcount);
+
 // records timing event k of the handle's current step (host side, fslbm_api.cu)
 int fslbm_mark(void* handle, int k);
 

@@ -27,7 +27,7 @@ namespace fsl {
 // one lane per cell; the liquid density is summed per warp.
 // ---------------------------------------------------------------------------
 template <int P>
-__global__ void __launch_bounds__(128, (P == P64 ? 4 : 8)) k_bulk(Par p, View<P> v, const int* __restrict__ seglist,
+__global__ void __launch_bounds__(128, 8) k_bulk(Par p, View<P> v, const int* __restrict__ seglist,
                                               const int* __restrict__ segcount) {
   pdl_begin();
   using R = typename Form<P>::R;
@@ -444,8 +444,12 @@ int launch_step_kernels(const Par& p, const View<P>& v, cudaStream_t st, int bul
       launched = true;
     }
   }
-  if (!launched && launch_k(k_bulk<P>, bulk_blocks, 128, 0, st, p, v, (const int*)seglist, (const int*)segcount))
-    return 1;
+  if constexpr (P == P64) {
+    if (launch_bulk_fixed(p, v, st, bulk_blocks, seglist, segcount)) return 1;
+  } else {
+    if (!launched && launch_k(k_bulk<P>, bulk_blocks, 128, 0, st, p, v, (const int*)seglist, (const int*)segcount))
+      return 1;
+  }
   if (timing_handle && fslbm_mark(timing_handle, 1)) return 1;
   if (geo && !side_geo && launch_k(kgeo, iface_blocks, 128, 0, st, p, v)) return 1;
   if (side_geo || side_if) {
