@@ -17,6 +17,7 @@
 // the launcher for one form, so that the forms compile in parallel.
 #pragma once
 #include "fslbm_dev.cuh"
+#include "fslbm_fixed.cuh"
 #include "fslbm_kernels.h"
 #include "fslbm_pull.cuh"
 
@@ -302,6 +303,127 @@ __device__ __forceinline__ double iface_cell(const Par& p, const View<P>& v, int
   return mm;
 }
 
+// c_q . a for an unrolled q
+template <class R>
+__device__ __forceinline__ R cdot(int q, const R (&a)[3]) {
+  R s = R(0);
+  if (cx(q)) s = cx(q) > 0 ? a[0] : -a[0];
+  if (cy(q)) s = cx(q) ? (cy(q) > 0 ? s + a[1] : s - a[1]) : (cy(q) > 0 ? a[1] : -a[1]);
+  if (cz(q)) s = (cx(q) || cy(q)) ? (cz(q) > 0 ? s + a[2] : s - a[2]) : (cz(q) > 0 ? a[2] : -a[2]);
+  return s;
+}
+
+// The FP64 form's default interface cell.  Its FP64 pipe (two operations a
+// cycle and SM) bounds it, so the arithmetic is laid out for few of them: the
+// equilibria, the non-equilibrium part and the quotient d / (n.c) are taken
+// once per link pair (a pair has at most one link with the FSL closure: its
+// upstream node must be fluid), both directions of a pair run the same
+// instructions on selected operands, and the collision is the fixed-point one.
+template <bool IN>
+__device__ __forceinline__ double iface_cell64(const Par& p, const View<P64>& v, int li, long long i, int x, int y,
+                                               int z, bool& fill, bool& empty) {
+  const size_t N = (size_t)p.N;
+  double own[19], f[19];
+#pragma unroll
+  for (int q = 0; q < 19; ++q) own[q] = v.fin[(size_t)q * N + (size_t)i];
+  f[0] = own[0];
+  unsigned wallm, gasm, liqm;
+  int srcs[19];  // sources of the pull (only kept off the interior path)
+  pull_general<P64, IN>(p, v, x, y, z, f, wallm, gasm, &liqm, IN ? nullptr : srcs);
+  const long long sy = p.nx, sz = (long long)p.nx * p.ny;
+  const double phic = v.phin[i];
+  double dm = 0.0;  // mass exchange (Sec. 2.3), twice its value
+  if (!p.freeze) {
+#pragma unroll
+    for (int q = 1; q < 19; ++q) {
+      if ((wallm | gasm) & (1u << q)) continue;
+      const long long sq = IN ? FSL_CK(p, i - (cx(q) + sy * cy(q) + sz * cz(q)), p.N) : (long long)srcs[q];
+      const double phs = v.phin[sq];
+      dm += ((liqm & (1u << q)) ? 2.0 : phic + phs) * (f[q] - own[inv(q)]);
+    }
+    dm *= 0.5;
+  }
+  if (wallm) wall_links<P64>(p, v, i, wallm, gasm, own, f);
+  if (gasm) {
+    double n[3] = {0.0, 0.0, 0.0}, d = 0.0, rb = p.rho_G;
+    if (p.rule != 0 || p.sigma != 0.0) {
+      const size_t cap = (size_t)v.cap;
+      n[0] = v.geo[li];
+      n[1] = v.geo[cap + li];
+      n[2] = v.geo[2 * cap + li];
+      d = v.geo[3 * cap + li];
+      rb += 3.0 * p.sigma * v.geo[4 * cap + li];
+    }
+    double rt = own[0], j[3] = {0.0, 0.0, 0.0};
+#pragma unroll
+    for (int q = 1; q < 19; q += 2) {
+      const double s = own[q] + own[q + 1], e = own[q] - own[q + 1];
+      rt += s;
+      if (cx(q)) j[0] += cx(q) * e;
+      if (cy(q)) j[1] += cy(q) * e;
+      if (cz(q)) j[2] += cz(q) * e;
+    }
+    const double r0t = p.compressible ? rt : 1.0, r0b = p.compressible ? rb : 1.0;
+    double u[3];
+#pragma unroll
+    for (int a = 0; a < 3; ++a) u[a] = (p.compressible ? j[a] / rt : j[a]) - 0.5 * p.g[a];
+    const double usq = u[0] * u[0] + u[1] * u[1] + u[2] * u[2], nl = p.linear_eq ? 0.0 : 1.0;
+#pragma unroll
+    for (int q = 1; q < 19; q += 2) {
+      constexpr double w1 = 1.0 / 18.0, w7 = 1.0 / 36.0;
+      const double w = q <= 6 ? w1 : w7;
+      const int qb = q + 1;
+      const bool ga = (gasm >> q) & 1u, gb = (gasm >> qb) & 1u;
+      if (!(ga || gb)) continue;
+      // e^+ of both directions: w rho + 3/2 w rho_0 (3 (c.u)^2 - u.u)
+      const double cu = cdot<double>(q, u), k = nl * (4.5 * w * cu * cu - 1.5 * w * usq);
+      const double eb = w * rb + r0b * k;
+      const unsigned blocked = wallm | gasm;
+      // FSL (Table 1): the rebuilt population's own link (q from qb's gas) has a fluid upstream node
+      const bool fa = p.rule != 0 && ga && !((blocked >> qb) & 1u), fb = p.rule != 0 && gb && !((blocked >> q) & 1u);
+      double val = 0.0;
+      if (fa || fb) {
+        const double s = own[q] + own[qb];
+        const double nplus = (0.5 * s - (w * rt + r0t * k)) * p.inv_1plp;
+        const double op = fa ? own[qb] : own[q], fup = fa ? f[qb] : f[q];
+        const double cq = cdot<double>(q, n), cn = fa ? -cq : cq;
+        double dl = 0.5;
+        if (cn > 0.0) {
+          dl = d / cn;
+          dl = dl < p.delta_min ? p.delta_min : (dl > 1.0 ? 1.0 : dl);
+        }
+        val = 0.5 * s - fup + dl * (fup - op) + p.lam_p * (dl - 1.5) * nplus + eb;
+      }
+      const double ska = 2.0 * eb - own[qb], skb = 2.0 * eb - own[q];  // FSK, Eq. koerner
+      if (ga) f[q] = fa ? val : ska;
+      if (gb) f[qb] = fb ? val : skb;
+    }
+  }
+  double rho;
+  long long rf;
+  bool over;
+  if (collide_fixed(p, f, rf, over)) {
+    rho = double_of_fix(rf);
+  } else {
+    double ux, uy, uz;
+    collide<double>(p, f, rho, ux, uy, uz);
+    if (rho_bad<false>(rho)) atomicOr(v.err, ERRB_UNSTABLE);
+  }
+#pragma unroll
+  for (int q = 0; q < 19; ++q) v.fout[(size_t)q * N + (size_t)i] = f[q];
+  double mm = v.m[i];
+  if (!p.freeze) {
+    mm = mm + dm;
+    v.m[i] = mm;
+    v.phout[i] = mm / rho;
+    fill = mm > (1.0 + p.eps) * rho || ((p.cleanup & 1) && gasm == 0u);
+    empty = !fill && (mm < -p.eps * rho || ((p.cleanup & 2) && (wallm | gasm) == 0x7fffeu));
+    if (fill) v.mark[i] = MK_FILL;
+    else if (empty) v.mark[i] = MK_EMPTY;
+  }
+  return mm;
+}
+
 // the geometry of cells within 3 of a face (bounded: no periodic axis);
 // inlined, so that its Geo stays in registers (an out-of-line call measured
 // slower: the edge warps set the kernel's tail)
@@ -353,8 +475,9 @@ __global__ void __launch_bounds__(128) k_geom(Par p, View<P> v) {
 
 // EXT: the instance with the boundary shear-rate term, the extrapolated u_b
 // and the normal links (separate, so that the default instance carries none
-// of their code)
-template <int P, bool EXT>
+// of their code).  LEAN: the FP64 form's instance with few FP64 operations
+// (where the fixed-point collision applies)
+template <int P, bool EXT, bool LEAN = false>
 __global__ void __launch_bounds__(128, (EXT ? 2 : (P == P64 ? 3 : 5))) k_iface(Par p, View<P> v, int part_base) {
   pdl_begin();
   const int n_in = min(*((volatile int*)&v.cnt[0]), v.cap), n_edge = min(*((volatile int*)&v.cnt[6]), v.cap);
@@ -375,8 +498,14 @@ __global__ void __launch_bounds__(128, (EXT ? 2 : (P == P64 ? 3 : 5))) k_iface(P
       int x, y, z;
       coords(p, i, x, y, z);
       if (FSL_OK(p, !in3 || (x >= 3 && x < p.nx - 3 && y >= 3 && y < p.ny - 3 && z >= 3 && z < p.nz - 3))) {
-        const double mm = in3 ? iface_cell<P, true, EXT>(p, v, pos, i, x, y, z, fill, empty)
-                              : iface_cell<P, false, EXT>(p, v, pos, i, x, y, z, fill, empty);
+        double mm;
+        if constexpr (LEAN) {
+          mm = in3 ? iface_cell64<true>(p, v, pos, i, x, y, z, fill, empty)
+                   : iface_cell64<false>(p, v, pos, i, x, y, z, fill, empty);
+        } else {
+          mm = in3 ? iface_cell<P, true, EXT>(p, v, pos, i, x, y, z, fill, empty)
+                   : iface_cell<P, false, EXT>(p, v, pos, i, x, y, z, fill, empty);
+        }
         if (owned(p, x, y, z)) msum += mm;
       }
     }
@@ -419,9 +548,12 @@ int launch_step_kernels(const Par& p, const View<P>& v, cudaStream_t st, int bul
   auto kgeo = p.elvira ? (p.sigma != 0.0 ? k_geom<P, true, true> : k_geom<P, false, true>)
                        : (p.sigma != 0.0 ? k_geom<P, true, false> : k_geom<P, false, false>);
   auto kif = (p.stress || p.ub_extrap || p.recon_nc) ? k_iface<P, true> : k_iface<P, false>;
+  if constexpr (P == P64) {
+    if (p.fix_ok && !(p.stress || p.ub_extrap || p.recon_nc)) kif = k_iface<P, false, true>;
+  }
   const bool pairs = P != P64 && bulk_mode == BULK_PAIRS;
   const bool side_geo = geo && fork;
-  const bool side_if = pairs && fork;
+  const bool side_if = (pairs || P == P64) && fork;
   if (side_geo || side_if) {
     if (cudaEventRecord(fork->fork, st) != cudaSuccess) return 1;
     if (cudaStreamWaitEvent(fork->side, fork->fork, 0) != cudaSuccess) return 1;
