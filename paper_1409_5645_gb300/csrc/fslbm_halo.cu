@@ -130,6 +130,7 @@ extern "C" int fslbm_set_owned(fslbm_t* h, const int lo[3], const int hi[3]) {
     all = all && lo[a] == 0 && hi[a] == n[a];
   }
   p.owned_all = all ? 1 : 0;
+  fslbm_drop_graphs(h);
   return FSLBM_OK;
 }
 

@@ -57,7 +57,14 @@ struct fslbm {
   int forked;         // fork holds a stream and events
   int overlap;        // 1: the interface kernels run on the side stream beside the bulk kernel
   int fp64_chain;     // the steps of a differentiation: the FP64 form without the fixed-point collision (Par::fix_ok)
+  // steps captured as graphs (see fslbm_step): [fp64_chain][cur][0] one step, [..][1] GRAPH_STEPS steps
+  cudaGraphExec_t graph[2][2][2];
+  cudaStream_t capture;  // the capturing stream (created with the first graph), or NULL
+  int graph_off;         // a capture or a graph launch failed: steps are launched one kernel at a time
 };
+
+// the captured steps hold the parameters by value: to be called when they change
+void fslbm_drop_graphs(fslbm* h);
 
 
 template <int P>
