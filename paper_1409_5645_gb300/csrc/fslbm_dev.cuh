@@ -884,6 +884,60 @@ __device__ __noinline__ void elvira_plane(const Par& p, const uint8_t* __restric
   }
 }
 
+// The normal, plane offset and curvature from the Parker-Youngs normal G.n
+// (not normalised, nn its square), the heights G.H and G.closed.  kopen: the
+// curvature where the columns are open, or NULL to have it computed here.
+template <class R, bool SIG, bool ELV>
+__device__ __forceinline__ void geometry_finish(const Par& p, const uint8_t* __restrict__ flags,
+                                                const R* __restrict__ phin, int x, int y, int z, R phic, R nn,
+                                                const R* kopen, Geo<R>& G) {
+  R (&n)[3] = G.n;
+  R& d = G.d;
+  R& kap = G.kap;
+  R (&H)[9] = G.H;
+  const int a = G.a, b = G.b, s = G.s;
+  if (G.closed) {
+    R Hb = R(0.5) * (H[7] - H[1]);
+    R Hc = R(0.5) * (H[5] - H[3]);
+    R v0 = (a == 0) ? R(s) : ((b == 0) ? -Hb : -Hc);
+    R v1 = (a == 1) ? R(s) : ((b == 1) ? -Hb : -Hc);
+    R v2 = (a == 2) ? R(s) : ((b == 2) ? -Hb : -Hc);
+    if constexpr (sizeof(R) == 4) {
+      const R il = rsqrtf(v0 * v0 + v1 * v1 + v2 * v2);
+      n[0] = v0 * il; n[1] = v1 * il; n[2] = v2 * il;
+    } else {
+      const R il = R(1) / sqrt(v0 * v0 + v1 * v1 + v2 * v2);
+      n[0] = v0 * il; n[1] = v1 * il; n[2] = v2 * il;
+    }
+    R nabs = fabs(a == 0 ? n[0] : (a == 1 ? n[1] : n[2]));
+    d = nabs * (H[4] - R(3.5));
+    if (SIG && p.sigma != 0.0) {
+      R Hbb = H[7] - R(2) * H[4] + H[1];
+      R Hcc = H[5] - R(2) * H[4] + H[3];
+      R Hbc = R(0.25) * (H[8] - H[6] - H[2] + H[0]);
+      R q2 = R(1) + Hb * Hb + Hc * Hc;
+      R num = Hbb * (R(1) + Hc * Hc) + Hcc * (R(1) + Hb * Hb) - R(2) * Hb * Hc * Hbc;
+      kap = -num / (q2 * sqrt(q2));
+    }
+  } else {
+    if (SIG && p.sigma != 0.0) kap = kopen ? *kopen : curvature_open<R>(p, flags, phin, x, y, z, n[0], n[1], n[2], a);
+    if constexpr (ELV) {
+      R ne[3];
+      elvira_plane<R>(p, flags, phin, x, y, z, phic, n[0], n[1], n[2], ne, &d);
+      n[0] = ne[0]; n[1] = ne[1]; n[2] = ne[2];
+      return;
+    }
+    if constexpr (sizeof(R) == 4) {
+      const R il = rsqrtf(nn);
+      n[0] *= il; n[1] *= il; n[2] *= il;
+    } else {
+      const R il = R(1) / sqrt(nn);
+      n[0] *= il; n[1] *= il; n[2] *= il;
+    }
+    d = plic_offset<R>(n[0], n[1], n[2], phic);
+  }
+}
+
 // MODE 0: any cell (plain offsets when every stencil cell is inside the
 // lattice, else the general neighbour rule); 1: the caller knows every cell
 // within 3 is inside; 2: a lattice without periodic axes (a stencil cell past
@@ -999,46 +1053,176 @@ __device__ __forceinline__ void geometry(const Par& p, const uint8_t* __restrict
       H[(ib + 1) * 3 + (ic + 1)] = sum;
     }
   G.closed = closed;
-  if (closed) {
-    R Hb = R(0.5) * (H[7] - H[1]);
-    R Hc = R(0.5) * (H[5] - H[3]);
-    R v0 = (a == 0) ? R(s) : ((b == 0) ? -Hb : -Hc);
-    R v1 = (a == 1) ? R(s) : ((b == 1) ? -Hb : -Hc);
-    R v2 = (a == 2) ? R(s) : ((b == 2) ? -Hb : -Hc);
-    if constexpr (sizeof(R) == 4) {
-      const R il = rsqrtf(v0 * v0 + v1 * v1 + v2 * v2);
-      n[0] = v0 * il; n[1] = v1 * il; n[2] = v2 * il;
-    } else {
-      const R il = R(1) / sqrt(v0 * v0 + v1 * v1 + v2 * v2);
-      n[0] = v0 * il; n[1] = v1 * il; n[2] = v2 * il;
-    }
-    R nabs = fabs(a == 0 ? n[0] : (a == 1 ? n[1] : n[2]));
-    d = nabs * (H[4] - R(3.5));
-    if (SIG && p.sigma != 0.0) {
-      R Hbb = H[7] - R(2) * H[4] + H[1];
-      R Hcc = H[5] - R(2) * H[4] + H[3];
-      R Hbc = R(0.25) * (H[8] - H[6] - H[2] + H[0]);
-      R q2 = R(1) + Hb * Hb + Hc * Hc;
-      R num = Hbb * (R(1) + Hc * Hc) + Hcc * (R(1) + Hb * Hb) - R(2) * Hb * Hc * Hbc;
-      kap = -num / (q2 * sqrt(q2));
-    }
-  } else {
-    if (SIG && p.sigma != 0.0) kap = curvature_open<R>(p, flags, phin, x, y, z, n[0], n[1], n[2], a);
-    if constexpr (ELV) {
-      R ne[3];
-      elvira_plane<R>(p, flags, phin, x, y, z, phic, n[0], n[1], n[2], ne, &d);
-      n[0] = ne[0]; n[1] = ne[1]; n[2] = ne[2];
-      return;
-    }
-    if constexpr (sizeof(R) == 4) {
-      const R il = rsqrtf(nn);
-      n[0] *= il; n[1] *= il; n[2] *= il;
-    } else {
-      const R il = R(1) / sqrt(nn);
-      n[0] *= il; n[1] *= il; n[2] *= il;
-    }
-    d = plic_offset<R>(n[0], n[1], n[2], phic);
+  geometry_finish<R, SIG, ELV>(p, flags, phin, x, y, z, phic, nn, (const R*)nullptr, G);
+}
+
+// ---------------------------------------------------------------------------
+// The same geometry by a warp per cell: the samples of the stencil on the
+// lanes, the sums in the thread's order (a lane's or, for the columns, handed
+// on between three lanes), so the results are the thread's bit for bit.
+// ---------------------------------------------------------------------------
+// fill level of the cell at offset (dx, dy, dz) and its kind (in3: the whole
+// stencil is inside the lattice)
+template <class R>
+__device__ __forceinline__ R coop_level(const Par& p, const uint8_t* __restrict__ flags, const R* __restrict__ phin,
+                                        int x, int y, int z, bool in3, int i, int dx, int dy, int dz, uint8_t& kj) {
+  const long long j = in3 ? (long long)(i + dx + p.nx * (dy + p.ny * dz)) : nbr(p, x, y, z, dx, dy, dz);
+  const R raw = j >= 0 ? phin[j] : R(0);
+  kj = kind_at(flags, j);
+  if (kj == LIQ) return R(1);
+  return kj == IFC || (kj == GAS && p.freeze) ? raw : R(0);
+}
+
+// Parker-Youngs gradient around (x, y, z), whose own fill level is phic (on
+// every lane); component a is summed by lane a in the stencil's order
+template <class R>
+__device__ __forceinline__ void coop_gradient(const Par& p, const uint8_t* __restrict__ flags,
+                                              const R* __restrict__ phin, int x, int y, int z, bool in3, int i,
+                                              R phic, R& g0, R& g1, R& g2) {
+  const int lane = threadIdx.x & 31, t = lane < 27 ? lane : 13;
+  uint8_t kj;
+  R v = coop_level<R>(p, flags, phin, x, y, z, in3, i, t % 3 - 1, (t / 3) % 3 - 1, t / 9 - 1, kj);
+  if (kj == WALL) v = phic;
+  R acc = R(0);
+#pragma unroll
+  for (int k = 0; k < 27; ++k) {
+    if (k == 13) continue;
+    const int dx = k % 3 - 1, dy = (k / 3) % 3 - 1, dz = k / 9 - 1;
+    const int ax = dx < 0 ? -dx : dx, ay = dy < 0 ? -dy : dy, az = dz < 0 ? -dz : dz;
+    const R w0 = R(dx * (2 - ay) * (2 - az)), w1 = R(dy * (2 - az) * (2 - ax)), w2 = R(dz * (2 - ax) * (2 - ay));
+    acc += (lane == 0 ? w0 : (lane == 1 ? w1 : w2)) * __shfl_sync(0xffffffffu, v, k);
   }
+  g0 = __shfl_sync(0xffffffffu, acc, 0);
+  g1 = __shfl_sync(0xffffffffu, acc, 1);
+  g2 = __shfl_sync(0xffffffffu, acc, 2);
+}
+
+// heights of the 3x3 columns along axis a (gas side s): column c on the lanes
+// c, c + 9, c + 18, which take its samples -3..-1, 0..1 and 2..3; returns
+// whether every column is closed.  stored (or NULL): the samples that are
+// stored fill levels, bit `lane` of word e the lane's e-th sample
+template <class R>
+__device__ __forceinline__ bool coop_columns(const Par& p, const uint8_t* __restrict__ flags,
+                                             const R* __restrict__ phin, int x, int y, int z, bool in3, int i, int a,
+                                             int s, R (&H)[9], unsigned* stored = nullptr) {
+  const unsigned FULL = 0xffffffffu;
+  const int lane = threadIdx.x & 31, g = lane / 9, c = lane - 9 * g;
+  const int b = a == 0 ? 1 : 0;
+  const int ib = c / 3 - 1, ic = c % 3 - 1;
+  R v[3];
+  bool bad = false;
+#pragma unroll
+  for (int e = 0; e < 3; ++e) {
+    const bool use = g < 3 && (e < 2 || g == 0);
+    const int k = g == 0 ? e - 3 : (g == 1 ? e : e + 2);
+    v[e] = R(0);
+    bool keeps = false;
+    if (use) {
+      uint8_t kj;
+      const int ox = a == 0 ? k : (b == 0 ? ib : ic), oy = a == 1 ? k : (b == 1 ? ib : ic), oz = a == 2 ? k : ic;
+      v[e] = coop_level<R>(p, flags, phin, x, y, z, in3, i, ox, oy, oz, kj);
+      bad = bad || kj == WALL;
+      if (k == -3) bad = bad || !(s > 0 ? kj == LIQ : kj == GAS);
+      if (k == 3) bad = bad || !(s > 0 ? kj == GAS : kj == LIQ);
+      keeps = kj == IFC || (kj == GAS && p.freeze);
+    }
+    if (stored) stored[e] = __ballot_sync(FULL, keeps);
+  }
+  R sum = (v[0] + v[1]) + v[2];
+  R below = __shfl_sync(FULL, sum, lane >= 9 ? lane - 9 : lane);
+  if (g == 1) sum = (below + v[0]) + v[1];
+  below = __shfl_sync(FULL, sum, lane >= 9 ? lane - 9 : lane);
+  if (g == 2) sum = (below + v[0]) + v[1];
+#pragma unroll
+  for (int m = 0; m < 9; ++m) H[m] = __shfl_sync(FULL, sum, 18 + m);
+  return __ballot_sync(FULL, bad) == 0u;
+}
+
+// curvature from nine column heights
+template <class R>
+__device__ __forceinline__ R heights_curvature(const R (&H)[9]) {
+  const R Hb = R(0.5) * (H[7] - H[1]);
+  const R Hc = R(0.5) * (H[5] - H[3]);
+  const R Hbb = H[7] - R(2) * H[4] + H[1];
+  const R Hcc = H[5] - R(2) * H[4] + H[3];
+  const R Hbc = R(0.25) * (H[8] - H[6] - H[2] + H[0]);
+  const R q2 = R(1) + Hb * Hb + Hc * Hc;
+  const R num = Hbb * (R(1) + Hc * Hc) + Hcc * (R(1) + Hb * Hb) - R(2) * Hb * Hc * Hbc;
+  return -num / (q2 * sqrt(q2));
+}
+
+// curvature_open by a warp
+template <class R>
+__device__ __noinline__ R coop_curvature_open(const Par& p, const uint8_t* __restrict__ flags,
+                                              const R* __restrict__ phin, int x, int y, int z, bool in3, int i, R n0,
+                                              R n1, R n2, int a) {
+  const R nv[3] = {n0, n1, n2};
+  int ax0 = (a + 1) % 3, ax1 = (a + 2) % 3;
+  const R v0 = ax0 == 0 ? n0 : (ax0 == 1 ? n1 : n2), v1 = ax1 == 0 ? n0 : (ax1 == 1 ? n1 : n2);
+  const bool swap = fabs(v1) > fabs(v0);
+#pragma unroll 1
+  for (int t = 0; t < 2; ++t) {
+    const bool second = (t == 1) != swap;
+    R H[9];
+    if (coop_columns<R>(p, flags, phin, x, y, z, in3, i, second ? ax1 : ax0, (second ? v1 : v0) > R(0) ? 1 : -1, H))
+      return heights_curvature<R>(H);
+  }
+  const R l0 = sqrt(nv[0] * nv[0] + nv[1] * nv[1] + nv[2] * nv[2]);
+  R div = R(0);
+#pragma unroll 1
+  for (int d = 0; d < 3; ++d) {
+    R comp[2];
+#pragma unroll
+    for (int sg = 0; sg < 2; ++sg) {
+      const int e = sg ? 1 : -1, ox = d == 0 ? e : 0, oy = d == 1 ? e : 0, oz = d == 2 ? e : 0;
+      const long long j = nbr(p, x, y, z, ox, oy, oz);
+      R m0 = n0, m1 = n1, m2 = n2, lm = l0;
+      if (j >= 0 && kind_at(flags, j) != WALL) {
+        uint8_t kc;
+        const R pc = fill_at<R>(p, flags, phin, j, kc);
+        R g0, g1, g2;
+        coop_gradient<R>(p, flags, phin, x + ox, y + oy, z + oz, in3, (int)j, pc, g0, g1, g2);
+        const R l = sqrt(g0 * g0 + g1 * g1 + g2 * g2);
+        if (l > R(1e-12)) {
+          m0 = -g0; m1 = -g1; m2 = -g2; lm = l;
+        }
+      }
+      comp[sg] = (d == 0 ? m0 : (d == 1 ? m1 : m2)) / lm;
+    }
+    div += R(0.5) * (comp[1] - comp[0]);
+  }
+  return div;
+}
+
+// The stencil's part of a cell's geometry by a warp (every lane gets it):
+// Parker-Youngs normal, heights, closed; false: no normal.  kopen receives the
+// curvature of open columns (SIG)
+template <class R, bool SIG>
+__device__ __forceinline__ bool coop_stencil(const Par& p, const uint8_t* __restrict__ flags,
+                                             const R* __restrict__ phin, int x, int y, int z, bool in3, int i, R phic,
+                                             R& nn, R& kopen, Geo<R>& G, unsigned* stored = nullptr) {
+  R g0, g1, g2;
+  coop_gradient<R>(p, flags, phin, x, y, z, in3, i, phic, g0, g1, g2);
+  G.n[0] = -g0; G.n[1] = -g1; G.n[2] = -g2;
+  G.kap = R(0);
+  G.d = R(0);
+  // (rounded as the thread's: where two components of the normal tie, its last
+  // bit decides the sign of n.c and with it a link fraction)
+  nn = fx_fma(G.n[2], G.n[2], fx_fma(G.n[0], G.n[0], fx_mul(G.n[1], G.n[1])));
+  kopen = R(0);
+  G.ok = nn > R(1e-24);
+  if (!G.ok) return false;
+  int a = 0;
+  R na = fabs(G.n[0]);
+  if (fabs(G.n[1]) > na) { a = 1; na = fabs(G.n[1]); }
+  if (fabs(G.n[2]) > na) { a = 2; }
+  G.a = a;
+  G.b = a == 0 ? 1 : 0;
+  G.s = (a == 0 ? G.n[0] : (a == 1 ? G.n[1] : G.n[2])) > R(0) ? 1 : -1;
+  G.closed = coop_columns<R>(p, flags, phin, x, y, z, in3, i, a, G.s, G.H, stored);
+  if (SIG && p.sigma != 0.0 && !G.closed)
+    kopen = coop_curvature_open<R>(p, flags, phin, x, y, z, in3, i, G.n[0], G.n[1], G.n[2], a);
+  return true;
 }
 
 // Fixed-order sum of chunk b of in[0, n) by the calling block of 256 threads:

@@ -83,6 +83,65 @@ __device__ __forceinline__ void pull_general(const Par& p, const View<P>& v, int
   if (liqm) *liqm = lm;
 }
 
+// The sources x - c_q of a cell's pull, -1 past a non-periodic face: each axis'
+// three neighbour coordinates (the x wrap shifts z) are taken once and a source
+// is the sum of three of them.  (nbr() unrolled 18 times is over a thousand
+// instructions.)
+__device__ __forceinline__ void pull_sources(const Par& p, int x, int y, int z, int (&srcs)[19]) {
+  int xo[3], yo[3], zo[3][3];
+  bool xv[3], yv[3], zv[3][3];
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    int X = x + k - 1, Y = y + k - 1, sh = 0;
+    if (p.px) {
+      if (X < 0) { X += p.nx; sh = p.zshift; }
+      else if (X >= p.nx) { X -= p.nx; sh = -p.zshift; }
+    }
+    if (p.py) Y += Y < 0 ? p.ny : (Y >= p.ny ? -p.ny : 0);
+    xo[k] = X;
+    xv[k] = (unsigned)X < (unsigned)p.nx;
+    yo[k] = Y * p.nx;
+    yv[k] = (unsigned)Y < (unsigned)p.ny;
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      int Z = z + c - 1 + sh;
+      if (p.pz) Z += Z < 0 ? p.nz : (Z >= p.nz ? -p.nz : 0);
+      zv[k][c] = (unsigned)Z < (unsigned)p.nz;
+      zo[k][c] = Z * (p.nx * p.ny);
+    }
+  }
+  srcs[0] = xo[1] + yo[1] + zo[1][1];
+#pragma unroll
+  for (int q = 1; q < 19; ++q) {
+    const int ka = 1 - cx(q), kb = 1 - cy(q), kc = 1 - cz(q);
+    srcs[q] = xv[ka] && yv[kb] && zv[ka][kc] ? xo[ka] + yo[kb] + zo[ka][kc] : -1;
+  }
+}
+
+// The pull of a cell that may lie on a face, for the interface kernel's edge
+// cells and the bulk kernels' out-of-line cells, which a warp meets one at a
+// time: sources from pull_sources, kinds and populations loaded together
+// (pull_general loads a population after its source's kind).
+template <int P>
+__device__ __forceinline__ void pull_table(const Par& p, const View<P>& v, int x, int y, int z,
+                                           typename Form<P>::R (&f)[19], unsigned& wallm, unsigned& gasm,
+                                           unsigned& liqm, int (&srcs)[19]) {
+  const size_t N = (size_t)p.N;
+  pull_sources(p, x, y, z, srcs);
+  wallm = gasm = liqm = 0u;
+#pragma unroll
+  for (int q = 1; q < 19; ++q) {
+    const bool in = srcs[q] >= 0;
+    const int s = in ? srcs[q] : 0;
+    const uint8_t ks = in ? (uint8_t)(v.flags[s] & KIND) : (uint8_t)WALL;
+    const typename Form<P>::R fq = ldq<P>(v.fin, (size_t)q * N + (size_t)s, q);
+    f[q] = is_fluid(ks) ? fq : typename Form<P>::R(0);
+    if (ks == LIQ) liqm |= 1u << q;
+    else if (ks == WALL) wallm |= 1u << q;
+    else if (ks != IFC) gasm |= 1u << q;
+  }
+}
+
 // Wall closure for the links in wallm (needs the cell's own f~ and the
 // pulled values): half-way bounce-back f_q = f~_p(x), p = qbar, or CLI with
 // kappa = (1 - 2 dw)/(1 + 2 dw): f_q = f~_p(x) + kappa (f~_p(x - c_p) - f~_q(x)),

@@ -24,9 +24,10 @@ __device__ __forceinline__ void general_cell(const Par& p, const View<P>& v, lon
                                              typename Form<P>::R (&f)[19]) {
   using R = typename Form<P>::R;
   const size_t N = (size_t)p.N;
-  unsigned wallm, gasm;
+  unsigned wallm, gasm, liqm;
+  int srcs[19];
   f[0] = ld<P, 0>(v.fin, (size_t)i);
-  pull_general<P>(p, v, x, y, z, f, wallm, gasm);
+  pull_table<P>(p, v, x, y, z, f, wallm, gasm, liqm, srcs);
   if (gasm) atomicOr(v.err, ERRB_STATE);  // liquid must not touch gas
   wallm |= gasm;
   if (wallm) {

@@ -157,7 +157,8 @@ __device__ __forceinline__ double iface_cell(const Par& p, const View<P>& v, int
   f[0] = own[0];
   unsigned wallm, gasm, liqm;
   int srcs[19];  // sources of the pull (only kept off the interior path)
-  pull_general<P, IN>(p, v, x, y, z, f, wallm, gasm, &liqm, IN ? nullptr : srcs);
+  if constexpr (IN) pull_general<P, true>(p, v, x, y, z, f, wallm, gasm, &liqm);
+  else pull_table<P>(p, v, x, y, z, f, wallm, gasm, liqm, srcs);
   const long long sy = p.nx, sz = (long long)p.nx * p.ny;
   const R phic = v.phin[i];
   // mass exchange (Sec. 2.3) with the pulled values, before any rebuild
@@ -329,7 +330,8 @@ __device__ __forceinline__ double iface_cell64(const Par& p, const View<P64>& v,
   f[0] = own[0];
   unsigned wallm, gasm, liqm;
   int srcs[19];  // sources of the pull (only kept off the interior path)
-  pull_general<P64, IN>(p, v, x, y, z, f, wallm, gasm, &liqm, IN ? nullptr : srcs);
+  if constexpr (IN) pull_general<P64, true>(p, v, x, y, z, f, wallm, gasm, &liqm);
+  else pull_table<P64>(p, v, x, y, z, f, wallm, gasm, liqm, srcs);
   const long long sy = p.nx, sz = (long long)p.nx * p.ny;
   const double phic = v.phin[i];
   double dm = 0.0;  // mass exchange (Sec. 2.3), twice its value
@@ -424,52 +426,76 @@ __device__ __forceinline__ double iface_cell64(const Par& p, const View<P64>& v,
   return mm;
 }
 
-// the geometry of cells within 3 of a face (bounded: no periodic axis);
-// inlined, so that its Geo stays in registers (an out-of-line call measured
-// slower: the edge warps set the kernel's tail)
-template <class R, bool BOUNDED, bool SIG, bool ELV>
-__device__ __forceinline__ void geometry_edge(const Par& p, const uint8_t* __restrict__ flags,
-                                           const R* __restrict__ phin, int x, int y, int z, R phic, Geo<R>& G) {
-  geometry<R, BOUNDED ? 2 : 0, SIG, ELV>(p, flags, phin, x, y, z, phic, G);
-}
-
 // ---------------------------------------------------------------------------
 // k_geom: plane (normal, offset) and curvature of every listed interface cell
-// from phi(t) (Sec. 2.2, Sec. 5), one thread per cell, into v.geo; kept apart
-// from k_iface so that each kernel holds fewer registers and less code.
+// from phi(t) (Sec. 2.2, Sec. 5) into v.geo; kept apart from k_iface so that
+// each kernel holds fewer registers and less code.
+//
+// A thread per cell has the higher throughput (its 89 samples and their sums
+// are about 1700 instructions for 32 cells) but is a chain of that length,
+// 25 to 35 us however few cells there are; a warp per cell spends about 550
+// instructions on one cell and is done with it in 3 to 5 us.  So each end of
+// the list, the interior cells and the edge cells (within 3 of a face, whose
+// samples need the neighbour rule), takes a thread per cell above
+// geom_warp_max cells and a warp per cell up to it; in FP64 the line is lower,
+// as a warp's finish holds the FP64 pipe as long for one cell as for 32.
+// Alone, with warm caches, thread -> warp: 16 FP64 cells of a 4x4x32 film 94
+// -> 13 us, 12.7 k FP32 cells of a 128x64x64 splash 28 -> 16 us, 17.4 k cells
+// with curvature of a 128^3 FP16 wave 93 -> 33 us; 57 k FP64 cells by threads
+// 55 us.
 // ---------------------------------------------------------------------------
+template <int P>
+constexpr int geom_warp_max() { return P == P64 ? 2432 : 49152; }
 // SIG: the instance that also computes the curvature (surface tension); ELV:
 // the one with the ELVIRA normal where the height columns are open
 template <int P, bool SIG, bool ELV>
 __global__ void __launch_bounds__(128) k_geom(Par p, View<P> v) {
   pdl_begin();
   using R = typename Form<P>::R;
-  const int n_in = min(*((volatile int*)&v.cnt[0]), v.cap), n_edge = min(*((volatile int*)&v.cnt[6]), v.cap);
-  const int count = min(n_in + n_edge, v.cap);
+  const int n_in = min(*((volatile int*)&v.cnt[0]), v.cap), n_edge = min(*((volatile int*)&v.cnt[6]), v.cap - n_in);
   const size_t cap = (size_t)v.cap;
-  for (int li = blockIdx.x * blockDim.x + threadIdx.x; li < count; li += gridDim.x * blockDim.x) {
-    const bool in3 = li < n_in;  // interior cells at the front, edge cells at the back
-    const int pos = in3 ? li : v.cap - 1 - (li - n_in);
+  auto put = [&](int pos, const Geo<R>& G) {
+    v.geo[pos] = G.ok ? G.n[0] : R(0);
+    v.geo[cap + pos] = G.ok ? G.n[1] : R(0);
+    v.geo[2 * cap + pos] = G.ok ? G.n[2] : R(0);
+    v.geo[3 * cap + pos] = G.d;
+    v.geo[4 * cap + pos] = G.kap;
+  };
+  // interior cells at the front of the list, edge cells at the back
+  const int t_in = n_in > geom_warp_max<P>() ? n_in : 0, t_edge = n_edge > geom_warp_max<P>() ? n_edge : 0;
+  for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < t_in + t_edge; e += gridDim.x * blockDim.x) {
+    const bool in3 = e < t_in;
+    const int pos = in3 ? e : v.cap - 1 - (e - t_in);
     const long long i = FSL_CK(p, v.ilist[pos], p.N);
     int x, y, z;
     coords(p, i, x, y, z);
     if (!FSL_OK(p, !in3 || (x >= 3 && x < p.nx - 3 && y >= 3 && y < p.ny - 3 && z >= 3 && z < p.nz - 3))) continue;
     const R phic = v.phin[i];
-    R o[5];
-    if (in3) {
-      Geo<R> G;  // (in registers)
-      geometry<R, 1, SIG, ELV>(p, v.flags, v.phin, x, y, z, phic, G);
-      o[0] = G.ok ? G.n[0] : R(0); o[1] = G.ok ? G.n[1] : R(0); o[2] = G.ok ? G.n[2] : R(0);
-      o[3] = G.d; o[4] = G.kap;
-    } else {
-      Geo<R> G;
-      if (!p.px && !p.py && !p.pz) geometry_edge<R, true, SIG, ELV>(p, v.flags, v.phin, x, y, z, phic, G);
-      else geometry_edge<R, false, SIG, ELV>(p, v.flags, v.phin, x, y, z, phic, G);
-      o[0] = G.ok ? G.n[0] : R(0); o[1] = G.ok ? G.n[1] : R(0); o[2] = G.ok ? G.n[2] : R(0);
-      o[3] = G.d; o[4] = G.kap;
+    Geo<R> G;  // (in registers)
+    if (in3) geometry<R, 1, SIG, ELV>(p, v.flags, v.phin, x, y, z, phic, G);
+    else if (!p.px && !p.py && !p.pz) geometry<R, 2, SIG, ELV>(p, v.flags, v.phin, x, y, z, phic, G);
+    else geometry<R, 0, SIG, ELV>(p, v.flags, v.phin, x, y, z, phic, G);
+    put(pos, G);
+  }
+  // a warp per cell, from the grid's last warps on
+  const int w_in = n_in - t_in, nc = w_in + n_edge - t_edge;
+  const int lane = threadIdx.x & 31, warps = (gridDim.x * blockDim.x) >> 5;
+  const int wid = warps - 1 - (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
+  for (int e = wid; e < nc; e += warps) {
+    const bool in3 = e < w_in;
+    const int pos = in3 ? e : v.cap - 1 - (e - w_in);
+    const long long i = FSL_CK(p, v.ilist[pos], p.N);
+    int x, y, z;
+    coords(p, i, x, y, z);
+    if (!FSL_OK(p, !in3 || (x >= 3 && x < p.nx - 3 && y >= 3 && y < p.ny - 3 && z >= 3 && z < p.nz - 3))) continue;
+    const R phic = v.phin[i];
+    Geo<R> G;
+    R nn, kopen;
+    const bool ok = coop_stencil<R, SIG>(p, v.flags, v.phin, x, y, z, in3, (int)i, phic, nn, kopen, G);
+    if (lane == 0) {
+      if (ok) geometry_finish<R, SIG, ELV>(p, v.flags, v.phin, x, y, z, phic, nn, &kopen, G);
+      put(pos, G);
     }
-#pragma unroll
-    for (int k = 0; k < 5; ++k) v.geo[k * cap + pos] = o[k];
   }
 }
 
