@@ -105,6 +105,20 @@ void fslbm_free_adjoint(fslbm* h) {
   h->adj = nullptr;
 }
 
+// A new state ends a differentiation.  Its buffers (some twenty allocations,
+// up to ADJ_KEEP_BYTES) stay with the handle for the next one of the same
+// window: allocating and freeing them was most of a short differentiation of a
+// 128x64x64 lattice.  Larger ones are given back at once.
+constexpr size_t ADJ_KEEP_BYTES = (size_t)2 << 30;
+void fslbm_end_adjoint(fslbm* h) {
+  if (!h->adj) return;
+  if (h->adj->bytes > ADJ_KEEP_BYTES) {
+    fslbm_free_adjoint(h);
+    return;
+  }
+  h->adj->ready = h->adj->live = false;
+}
+
 static bool amalloc(AdjointState* A, void** p, size_t bytes) {
   if (cudaMalloc(p, bytes ? bytes : 16) != cudaSuccess) {
     *p = nullptr;
@@ -143,20 +157,27 @@ extern "C" int fslbm_adjoint_forward(fslbm_t* h, int nsteps, int K, int objectiv
   if (h->par.recon_nc) return adj_fail(h, FSLBM_ERR_ARG, "adjoint needs the gas links only (recon_nc = 0)");
   if (h->par.excess_split) return adj_fail(h, FSLBM_ERR_ARG, "adjoint needs the equal excess split");
   if (h->par.elvira) return adj_fail(h, FSLBM_ERR_ARG, "adjoint needs the Parker-Youngs plane fit (elvira = 0)");
-  fslbm_free_adjoint(h);
-  AdjointState* A = new AdjointState();
-  h->adj = A;
+  const int nck = (nsteps + K - 1) / K;
+  // the buffers of an ended differentiation of the same window serve again
+  const bool kept = h->adj && !h->adj->live && h->adj->nck == nck && h->adj->K == K;
+  if (!kept) {
+    fslbm_free_adjoint(h);
+    h->adj = new AdjointState();
+  }
+  AdjointState* A = h->adj;
   const size_t N = (size_t)h->par.N;
   A->nsteps = nsteps;
   A->K = K;
   A->objective = objective;
-  A->nck = (nsteps + K - 1) / K;
+  A->nck = nck;
+  A->live = true;
+  A->ready = false;
   const size_t sb = h->prec == FSLBM_F64 ? 8 : (h->prec == FSLBM_F32 ? 4 : 2);
   A->fbytes = 19 * N * sb;
   A->rbytes = N * (h->prec == FSLBM_F64 ? 8 : 4);
-  bool ok = amalloc(A, &A->ck_f, A->fbytes * A->nck) && amalloc(A, (void**)&A->ck_m, N * 8 * A->nck) &&
+  bool ok = kept || (amalloc(A, &A->ck_f, A->fbytes * A->nck) && amalloc(A, (void**)&A->ck_m, N * 8 * A->nck) &&
             amalloc(A, &A->ck_phi, A->rbytes * A->nck) && amalloc(A, (void**)&A->ck_flags, N * A->nck) &&
-            amalloc(A, (void**)&A->red, 64);
+            amalloc(A, (void**)&A->red, ADJ_RED_DOUBLES * 8));
   if (!ok) {
     fslbm_free_adjoint(h);
     return adj_fail(h, FSLBM_ERR_OOM, "adjoint checkpoint allocation");
@@ -257,7 +278,7 @@ extern "C" int fslbm_adjoint_backward(fslbm_t* h, double* dJ_dnu, double dJ_dg[3
 
 extern "C" int fslbm_adjoint_stats(fslbm_t* h, double* fwd_ms_per_step, double* adj_ms_per_step,
                                    size_t* peak_bytes) {
-  if (!h || !h->adj) return FSLBM_ERR_ARG;
+  if (!h || !h->adj || !h->adj->live) return FSLBM_ERR_ARG;
   if (fwd_ms_per_step) *fwd_ms_per_step = h->adj->fwd_ms;
   if (adj_ms_per_step) *adj_ms_per_step = h->adj->adj_ms;
   if (peak_bytes) *peak_bytes = h->adj->bytes + h->bytes;

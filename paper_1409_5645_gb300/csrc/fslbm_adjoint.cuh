@@ -6,6 +6,7 @@
 #include <stdio.h>
 
 #include "fslbm_adjoint.h"
+#include "fslbm_pull.cuh"
 
 using namespace fsl;
 
@@ -64,6 +65,20 @@ template <class A>
 __device__ __forceinline__ void deplus_du(const Par& p, int q, A ux, A uy, A uz, A g, A (&ub)[3]) {
   if (p.linear_eq) return;
   A w = q == 0 ? A(1.0) / A(3.0) : (q <= 6 ? A(1.0) / A(18.0) : A(1.0) / A(36.0));
+  if constexpr (sizeof(A) == 8) {
+    A cu = A(0);
+    if (cx(q)) cu = cx(q) > 0 ? ux : -ux;
+    if (cy(q)) cu = cy(q) > 0 ? cu + uy : cu - uy;
+    if (cz(q)) cu = cz(q) > 0 ? cu + uz : cu - uz;
+    const A t = g * w, t9 = A(9.0) * cu * t, t3 = A(3.0) * t;
+    ub[0] -= t3 * ux;
+    ub[1] -= t3 * uy;
+    ub[2] -= t3 * uz;
+    if (cx(q)) ub[0] += cx(q) * t9;
+    if (cy(q)) ub[1] += cy(q) * t9;
+    if (cz(q)) ub[2] += cz(q) * t9;
+    return;
+  }
   A cu = A(cx(q)) * ux + A(cy(q)) * uy + A(cz(q)) * uz;
   ub[0] += g * w * (A(9.0) * cu * cx(q) - A(3.0) * ux);
   ub[1] += g * w * (A(9.0) * cu * cy(q) - A(3.0) * uy);
@@ -75,7 +90,15 @@ __device__ __forceinline__ A eplus_d(const Par& p, int q, A rho, A ux, A uy, A u
   A w = q == 0 ? A(1.0) / A(3.0) : (q <= 6 ? A(1.0) / A(18.0) : A(1.0) / A(36.0));
   A e = w * rho;
   if (!p.linear_eq) {
-    A cu = A(cx(q)) * ux + A(cy(q)) * uy + A(cz(q)) * uz;
+    A cu;
+    if constexpr (sizeof(A) == 8) {  // (the same value; a zero component leaves no operation)
+      cu = A(0);
+      if (cx(q)) cu = cx(q) > 0 ? ux : -ux;
+      if (cy(q)) cu = cy(q) > 0 ? cu + uy : cu - uy;
+      if (cz(q)) cu = cz(q) > 0 ? cu + uz : cu - uz;
+    } else {
+      cu = A(cx(q)) * ux + A(cy(q)) * uy + A(cz(q)) * uz;
+    }
     e += w * A(1.5) * (A(3.0) * cu * cu - (ux * ux + uy * uy + uz * uz));
   }
   return e;
@@ -83,8 +106,82 @@ __device__ __forceinline__ A eplus_d(const Par& p, int q, A rho, A ux, A uy, A u
 
 // Reverse of the TRT collision (Eq. lbe2, rho_0 = 1) at pre-collision f with
 // output adjoint ab: adds to fb and to th (lambda_+, lambda_-, g).
+// In FP64 the pipe's two operations a cycle and SM are the bound: there the
+// terms of a link pair are formed once and the components that are zero leave
+// no operation (8x4x64 film, the liquid instance 34 -> 22 us).  The
+// non-equilibrium parts keep the expressions of the general form: near
+// equilibrium they are differences of nearly equal numbers, and the adjoint of
+// the viscosity is a sum over them (other roundings of theirs moved a film's
+// dJ/dnu by 2e-8).  The float form keeps all its expressions.
+__device__ __forceinline__ void collide_rev64(const Par& p, const double (&f)[19], const double (&ab)[19],
+                                              double (&fb)[19], double (&th)[5]) {
+  const double lp = p.lam_p, lm = p.lam_m;
+  double r = 0.0, jx = 0.0, jy = 0.0, jz = 0.0;
+  auto add = [](double (&v)[3], int q, double x) {
+    if (cx(q)) v[0] += cx(q) > 0 ? x : -x;
+    if (cy(q)) v[1] += cy(q) > 0 ? x : -x;
+    if (cz(q)) v[2] += cz(q) > 0 ? x : -x;
+  };
+  auto dot = [](const double (&v)[3], int q) {
+    double s = 0.0;
+    if (cx(q)) s = cx(q) > 0 ? v[0] : -v[0];
+    if (cy(q)) s = cy(q) > 0 ? s + v[1] : s - v[1];
+    if (cz(q)) s = cz(q) > 0 ? s + v[2] : s - v[2];
+    return s;
+  };
+#pragma unroll
+  for (int q = 0; q < 19; ++q) {
+    r += f[q];
+    if (cx(q)) jx += double(cx(q)) * f[q];
+    if (cy(q)) jy += double(cy(q)) * f[q];
+    if (cz(q)) jz += double(cz(q)) * f[q];
+  }
+  const double g0 = p.g[0], g1 = p.g[1], g2 = p.g[2], nl = p.linear_eq ? 0.0 : 1.0;
+  const double u[3] = {jx + 0.5 * g0, jy + 0.5 * g1, jz + 0.5 * g2};
+  const double v[3] = {jx - g0 / lm, jy - g1 / lm, jz - g2 / lm};
+  // rest population; dens: sum of w times the adjoints of e^+ (negated), for rho and the -3/2 w u.u part
+  const double np0 = f[0] - eplus_d<double>(p, 0, r, u[0], u[1], u[2]), npb0 = lp * ab[0];
+  th[0] += np0 * ab[0];
+  fb[0] += ab[0] + npb0;
+  double dens = (1.0 / 3.0) * npb0, ub[3] = {0.0, 0.0, 0.0}, vb[3] = {0.0, 0.0, 0.0};
+#pragma unroll
+  for (int q = 1; q < 19; q += 2) {
+    const int qb = q + 1;
+    const double w = q <= 6 ? 1.0 / 18.0 : 1.0 / 36.0;
+    const double cu = nl * dot(u, q), sp = ab[q] + ab[qb], sm = ab[q] - ab[qb];
+    const double ep = eplus_d<double>(p, q, r, u[0], u[1], u[2]), em = 3.0 * w * dot(v, q);
+    const double np = 0.5 * (f[q] + f[qb]) - ep, nm = 0.5 * (f[q] - f[qb]) - em;
+    const double npb = lp * sp, nmb = lm * sm;
+    th[0] += np * sp;
+    th[1] += nm * sm;
+    fb[q] += ab[q] + 0.5 * (npb + nmb);
+    fb[qb] += ab[qb] + 0.5 * (npb - nmb);
+    dens += w * npb;
+    add(ub, q, -9.0 * w * cu * npb);
+    add(vb, q, -3.0 * w * nmb);
+  }
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    ub[a] += 3.0 * nl * dens * u[a];
+    th[2 + a] += 0.5 * ub[a] - vb[a] * p.inv_lam_m;
+    ub[a] += vb[a];
+  }
+  th[1] += (g0 * vb[0] + g1 * vb[1] + g2 * vb[2]) / (lm * lm);
+  fb[0] -= dens;
+#pragma unroll
+  for (int q = 1; q < 19; q += 2) {
+    const double d = dot(ub, q);
+    fb[q] += d - dens;
+    fb[q + 1] -= d + dens;
+  }
+}
+
 template <class A>
 __device__ void collide_rev(const Par& p, const A (&f)[19], const A (&ab)[19], A (&fb)[19], A (&th)[5]) {
+  if constexpr (sizeof(A) == 8) {
+    collide_rev64(p, f, ab, fb, th);
+    return;
+  }
   const A lp = (A)p.lam_p, lm = (A)p.lam_m;
   const A g0 = (A)p.g[0], g1 = (A)p.g[1], g2 = (A)p.g[2];
   A r = 0, jx = 0, jy = 0, jz = 0;
@@ -199,7 +296,10 @@ static __device__ void plane_section(const double (&n)[3], double d, double& A, 
   int ord[12];
   for (int k = 0; k < np; ++k) {
     const double r0 = P[k][0] - m[0], r1 = P[k][1] - m[1], r2 = P[k][2] - m[2];
-    ang[k] = atan2(r0 * v[0] + r1 * v[1] + r2 * v[2], r0 * u[0] + r1 * u[1] + r2 * u[2]);
+    // a quantity that grows with the angle from -2 to 2 (no atan2: only the order counts)
+    const double s = r0 * v[0] + r1 * v[1] + r2 * v[2], t = r0 * u[0] + r1 * u[1] + r2 * u[2];
+    const double e = t / (fabs(s) + fabs(t));
+    ang[k] = __double_as_longlong(s) < 0 ? e - 1.0 : 1.0 - e;
     ord[k] = k;
   }
   for (int k = 1; k < np; ++k)  // insertion sort by angle
@@ -284,14 +384,68 @@ __device__ __noinline__ double plane_fit_adjoint(const Par& p, const uint8_t* __
 // does: moments rho - 1, the gas density rho_G - 1 in the rebuilt links; every
 // closure is affine in the populations with weights summing to one per link
 // pair, so only the densities that divide (phi = m / rho) take the 1 back).
+//
+// The interface instance in FP64 arithmetic runs as k_geom does: a warp
+// computes the geometry of its cells one after the other with the stencil on
+// its lanes (into shared memory), then takes a cell per lane; as few cells go
+// to a warp as keep four warps on an SM, where the FP64 pipe is the bound.
+// With the 89 samples and the neighbour rule on one thread, a chain of over ten
+// thousand instructions, 32 cells of an 8x4x64 film took 250 us (alone, cold
+// caches), 103 us so.  The float instance keeps a thread per cell: its open
+// cells' plane fits, thousands of instructions each, want full warps (12.7 k
+// cells of a 128x64x64 splash 192 us, spread thinly 388 us).
+template <class R>
+struct AdjGeo {
+  Geo<R> G;
+  unsigned stored[3];  // samples of the columns that are stored fill levels (coop_columns)
+};
+
 template <int P, bool IFCP, class A>
 __global__ void __launch_bounds__(128) k_adj_local(Par p, AdjView<P> a) {
   using R = typename Form<P>::R;
   constexpr bool SH = sizeof(A) == 4 && Form<P>::SH;
   const size_t N = (size_t)p.N;
   A th[5] = {0, 0, 0, 0, 0};
+  // COOP: the interface instance in FP64 arithmetic (see above)
+  constexpr bool COOP = IFCP && sizeof(A) == 8;
   const int nf = *a.nfl;
-  for (int li = blockIdx.x * blockDim.x + threadIdx.x; li < nf; li += gridDim.x * blockDim.x) {
+  const int lane = threadIdx.x & 31, warps = (gridDim.x * blockDim.x) >> 5;
+  const int wid = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  const int spread = min(warps, 152 * 4);
+  const int per = COOP ? min(max((nf + spread - 1) / spread, 1), 32) : 32;  // cells per warp and round
+  __shared__ AdjGeo<R> sgeo[COOP ? 128 : 1];
+  AdjGeo<R>* wgeo = COOP ? sgeo + (threadIdx.x & ~31) : sgeo;
+  for (int base = wid * per; base < nf; base += warps * per) {
+    if constexpr (COOP) {
+      __syncwarp();
+      if (p.rule != 0) {  // (FSK uses no geometry)
+        for (int k = 0; k < per && base + k < nf; ++k) {
+          const long long ik = FSL_CK(p, a.flist[base + k], p.N);
+          int xk, yk, zk;
+          coords(p, ik, xk, yk, zk);
+          bool gas = false;
+          if (lane >= 1 && lane < 19) {
+            const long long j = nbr(p, xk, yk, zk, cx(lane), cy(lane), cz(lane));
+            gas = j >= 0 && (a.flags[j] & KIND) == GAS;
+          }
+          if (__ballot_sync(0xffffffffu, gas) == 0u) continue;  // no gas link: not used
+          const bool in3 = xk >= 3 && xk < p.nx - 3 && yk >= 3 && yk < p.ny - 3 && zk >= 3 && zk < p.nz - 3;
+          const R ph = a.phi[ik];
+          Geo<R> G;
+          unsigned st[3] = {0u, 0u, 0u};
+          R nn, kopen;
+          const bool ok = coop_stencil<R, false>(p, a.flags, a.phi, xk, yk, zk, in3, (int)ik, ph, nn, kopen, G, st);
+          if (lane == 0) {
+            if (ok) geometry_finish<R, false, false>(p, a.flags, a.phi, xk, yk, zk, ph, nn, &kopen, G);
+            wgeo[k].G = G;
+            wgeo[k].stored[0] = st[0]; wgeo[k].stored[1] = st[1]; wgeo[k].stored[2] = st[2];
+          }
+        }
+      }
+      __syncwarp();
+    }
+    const int li = base + lane;
+    if (lane >= per || li >= nf) continue;
     const long long i = FSL_CK(p, a.flist[li], p.N);
     const uint8_t kc = IFCP ? (uint8_t)IFC : (uint8_t)LIQ;
     int x, y, z;
@@ -303,14 +457,26 @@ __global__ void __launch_bounds__(128) k_adj_local(Par p, AdjView<P> a) {
     int src[19];
     F[0] = own[0];
     src[0] = (int)i;
+    if constexpr (sizeof(A) == 8) {
+      pull_sources(p, x, y, z, src);
 #pragma unroll
-    for (int q = 1; q < 19; ++q) {
-      long long s = nbr(p, x, y, z, -cx(q), -cy(q), -cz(q));
-      src[q] = (int)s;
-      uint8_t ks = kind_at(a.flags, s);
-      if (is_fluid(ks)) F[q] = ld_adj<P, A>(a.f, q * N + s, q);
-      else if (ks == WALL) { wallm |= 1u << q; F[q] = A(0.0); }
-      else { gasm |= 1u << q; F[q] = A(0.0); }
+      for (int q = 1; q < 19; ++q) {
+        const uint8_t ks = src[q] < 0 ? (uint8_t)WALL : (uint8_t)(a.flags[src[q]] & KIND);
+        const A v = ld_adj<P, A>(a.f, q * N + (src[q] < 0 ? 0 : src[q]), q);
+        F[q] = is_fluid(ks) ? v : A(0.0);
+        if (ks == WALL) wallm |= 1u << q;
+        else if (!is_fluid(ks)) gasm |= 1u << q;
+      }
+    } else {
+#pragma unroll
+      for (int q = 1; q < 19; ++q) {
+        long long s = nbr(p, x, y, z, -cx(q), -cy(q), -cz(q));
+        src[q] = (int)s;
+        uint8_t ks = kind_at(a.flags, s);
+        if (is_fluid(ks)) F[q] = ld_adj<P, A>(a.f, q * N + s, q);
+        else if (ks == WALL) { wallm |= 1u << q; F[q] = A(0.0); }
+        else { gasm |= 1u << q; F[q] = A(0.0); }
+      }
     }
     if constexpr (!IFCP) gasm = 0u;  // (liquid cells have no gas neighbour)
 #pragma unroll
@@ -320,9 +486,9 @@ __global__ void __launch_bounds__(128) k_adj_local(Par p, AdjView<P> a) {
 #pragma unroll
     for (int q = 0; q < 19; ++q) {
       rt += own[q];
-      tx += cx(q) * own[q];
-      ty += cy(q) * own[q];
-      tz += cz(q) * own[q];
+      if (sizeof(A) == 4 || cx(q)) tx += cx(q) * own[q];
+      if (sizeof(A) == 4 || cy(q)) ty += cy(q) * own[q];
+      if (sizeof(A) == 4 || cz(q)) tz += cz(q) * own[q];
     }
     const A utx = tx - A(0.5) * (A)p.g[0], uty = ty - A(0.5) * (A)p.g[1], utz = tz - A(0.5) * (A)p.g[2];
     const bool ifc = kc == IFC;
@@ -359,13 +525,14 @@ __global__ void __launch_bounds__(128) k_adj_local(Par p, AdjView<P> a) {
       f[q] = val;
     }
     // free-surface closures (forward, keeping what the reverse needs)
-    Geo<R> G;
+    Geo<R> Gt;
+    const Geo<R>& G = COOP ? wgeo[lane].G : Gt;
     A dl[19], npl[19], et[19];
     bool fsl[19];
     const A lp = (A)p.lam_p, inv1 = (A)p.inv_1plp, dmin = (A)p.delta_min;
     const A rhoG = SH ? (A)(p.rho_G - 1.0) : (A)p.rho_G;  // (deviation of the gas density)
     if (gasm) {
-      geometry<R>(p, a.flags, a.phi, x, y, z, (R)phic, G);
+      if constexpr (!COOP) geometry<R>(p, a.flags, a.phi, x, y, z, (R)phic, Gt);
 #pragma unroll
       for (int q = 1; q < 19; ++q) {
         fsl[q] = false;
@@ -527,15 +694,20 @@ __global__ void __launch_bounds__(128) k_adj_local(Par p, AdjView<P> a) {
           const A hb = Hbar[(ib + 1) * 3 + (ic + 1)];
           if (hb == A(0.0)) continue;
           for (int k = -3; k <= 3; ++k) {
+            if constexpr (COOP) {  // (the lane and word of the sample in coop_columns)
+              const int g = k < 0 ? 0 : (k < 2 ? 1 : 2), e = k < 0 ? k + 3 : (k < 2 ? k : k - 2);
+              if (!((wgeo[lane].stored[e] >> ((ib + 1) * 3 + (ic + 1) + 9 * g)) & 1u)) continue;
+            }
             int o0 = (Ax == 0) ? k : ((B == 0) ? ib : ic);
             int o1 = (Ax == 1) ? k : ((B == 1) ? ib : ic);
             int o2 = (Ax == 2) ? k : ((B == 2) ? ib : ic);
             long long j = nbr(p, x, y, z, o0, o1, o2);
-            uint8_t kj = kind_at(a.flags, j);
-            if (kj == IFC || (kj == GAS && p.freeze)) {
-              if (j == i) phib_self += hb;
-              else atomicAdd(a.phibar_out + j, (double)hb);
+            if constexpr (!COOP) {
+              uint8_t kj = kind_at(a.flags, j);
+              if (!(kj == IFC || (kj == GAS && p.freeze))) continue;
             }
+            if (j == i) phib_self += hb;
+            else atomicAdd(a.phibar_out + j, (double)hb);
           }
         }
     }
@@ -546,7 +718,16 @@ __global__ void __launch_bounds__(128) k_adj_local(Par p, AdjView<P> a) {
     }
     // own moments: rho_t = sum f~, u_t = sum c f~ - g/2
 #pragma unroll
-    for (int q = 0; q < 19; ++q) ob[q] += rtb + cx(q) * utb[0] + cy(q) * utb[1] + cz(q) * utb[2];
+    for (int q = 0; q < 19; ++q) {
+      if constexpr (sizeof(A) == 8) {  // (no operation for a zero component)
+        ob[q] += rtb;
+        if (cx(q)) ob[q] += cx(q) * utb[0];
+        if (cy(q)) ob[q] += cy(q) * utb[1];
+        if (cz(q)) ob[q] += cz(q) * utb[2];
+      } else {
+        ob[q] += rtb + cx(q) * utb[0] + cy(q) * utb[1] + cz(q) * utb[2];
+      }
+    }
     th[2] -= A(0.5) * utb[0];
     th[3] -= A(0.5) * utb[1];
     th[4] -= A(0.5) * utb[2];
@@ -570,11 +751,12 @@ __global__ void k_adj_gather(Par p, const uint8_t* __restrict__ flags, const dou
   const int nl = cnt[0], ni = cnt[1];
   for (int li = blockIdx.x * blockDim.x + threadIdx.x; li < nl + ni; li += gridDim.x * blockDim.x) {
     const long long i = FSL_CK(p, li < nl ? liq[li] : ifc[li - nl], p.N);
-    int x, y, z;
+    int x, y, z, src[19];
     coords(p, i, x, y, z);
+    pull_sources(p, x, y, z, src);
 #pragma unroll
     for (int q = 1; q < 19; ++q) {
-      long long zc = nbr(p, x, y, z, cx(q), cy(q), cz(q));
+      const int zc = src[inv(q)];  // x + c_q
       if (zc < 0 || !is_fluid(flags[zc] & KIND)) continue;
       abar[q * N + i] += Pb[q * N + zc];
     }
@@ -583,9 +765,12 @@ __global__ void k_adj_gather(Par p, const uint8_t* __restrict__ flags, const dou
 
 // Objective on the stored state: red[0] = sum of the objective's terms,
 // red[1] = count (interface cells) or sum of phi (flux).
+// (a block's sums go to its slots of red, and the last block to finish adds
+// them up in order: an atomic per thread on the two results took 930 us on a
+// 128x64x64 lattice)
 template <int P>
-__global__ void k_objective(Par p, const uint8_t* flags, const typename Form<P>::S* f,
-                            const typename Form<P>::R* phi, int objective, double* red) {
+__global__ void __launch_bounds__(256) k_objective(Par p, const uint8_t* flags, const typename Form<P>::S* f,
+                                                   const typename Form<P>::R* phi, int objective, double* red) {
   const size_t N = (size_t)p.N;
   double s = 0.0, c = 0.0;
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < p.N;
@@ -602,8 +787,48 @@ __global__ void k_objective(Par p, const uint8_t* flags, const typename Form<P>:
     s += w * ux;
     c += w;
   }
-  atomicAdd(red, s);
-  atomicAdd(red + 1, c);
+  __shared__ double sh[2][8];
+  __shared__ bool last;
+  auto block_sum = [&](double a, double b) {  // on thread 0
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      a += __shfl_down_sync(0xffffffffu, a, o);
+      b += __shfl_down_sync(0xffffffffu, b, o);
+    }
+    __syncthreads();
+    if ((threadIdx.x & 31) == 0) {
+      sh[0][threadIdx.x >> 5] = a;
+      sh[1][threadIdx.x >> 5] = b;
+    }
+    __syncthreads();
+    s = c = 0.0;
+    if (threadIdx.x == 0)
+      for (int k = 0; k < 8; ++k) {
+        s += sh[0][k];
+        c += sh[1][k];
+      }
+  };
+  block_sum(s, c);
+  double* part = red + 8;
+  if (threadIdx.x == 0) {
+    part[2 * blockIdx.x] = s;
+    part[2 * blockIdx.x + 1] = c;
+    __threadfence();
+    last = atomicAdd(reinterpret_cast<unsigned*>(red + 2), 1u) == gridDim.x - 1;
+    __threadfence();
+  }
+  __syncthreads();
+  if (!last) return;
+  double a = 0.0, b = 0.0;
+  for (unsigned k = threadIdx.x; k < gridDim.x; k += 256) {
+    a += __ldcg(part + 2 * k);
+    b += __ldcg(part + 2 * k + 1);
+  }
+  block_sum(a, b);
+  if (threadIdx.x == 0) {
+    red[0] = s;
+    red[1] = c;
+  }
 }
 
 template <int P>
@@ -650,40 +875,44 @@ __global__ void __launch_bounds__(128) k_adj_init(Par p, const uint8_t* flags, c
     uint8_t k = flags[i] & KIND;
     dphi0[i] = 0.0;
     if (!is_fluid(k)) continue;
-    double ft[19], f0[19], ab[19], fb[19];
-    double r = 0, jx = 0, jy = 0, jz = 0;
+    double f0[19], ab[19], fb[19];
+    double r = 0.0;
 #pragma unroll
     for (int q = 0; q < 19; ++q) {
-      ft[q] = ldq_full<P>(f, q * N + i, q);
       ab[q] = abar[q * N + i];
       fb[q] = 0.0;
-      r += ft[q];
-      jx += cx(q) * ft[q];
-      jy += cy(q) * ft[q];
-      jz += cz(q) * ft[q];
-    }
-    // U = sum c f~ - g, u = U + g/2, v = U - g/lambda_-
-    const double Ux = jx - p.g[0], Uy = jy - p.g[1], Uz = jz - p.g[2];
-    const double ux = Ux + 0.5 * p.g[0], uy = Uy + 0.5 * p.g[1], uz = Uz + 0.5 * p.g[2];
-    const double vx = Ux - p.g[0] / p.lam_m, vy = Uy - p.g[1] / p.lam_m, vz = Uz - p.g[2] / p.lam_m;
-    f0[0] = eplus_d(p, 0, r, ux, uy, uz) + (ft[0] - eplus_d(p, 0, r, ux, uy, uz)) / (1.0 + p.lam_p);
-#pragma unroll
-    for (int q = 1; q < 19; q += 2) {
-      const int qb = q + 1;
-      double w = q <= 6 ? 1.0 / 18.0 : 1.0 / 36.0;
-      double ep = eplus_d(p, q, r, ux, uy, uz);
-      double em = 3.0 * w * (cx(q) * vx + cy(q) * vy + cz(q) * vz);
-      double fp = ep + (0.5 * (ft[q] + ft[qb]) - ep) / (1.0 + p.lam_p);
-      double fm = em + (0.5 * (ft[q] - ft[qb]) - em) / (1.0 + p.lam_m);
-      f0[q] = fp + fm;
-      f0[qb] = fp - fm;
     }
     if (f0keep) {  // the initial populations as set, in FP64
-      r = 0.0;
 #pragma unroll
       for (int q = 0; q < 19; ++q) {
         f0[q] = f0keep[(size_t)q * N + i];
         r += f0[q];
+      }
+    } else {  // from the collided ones
+      double ft[19], jx = 0.0, jy = 0.0, jz = 0.0;
+#pragma unroll
+      for (int q = 0; q < 19; ++q) {
+        ft[q] = ldq_full<P>(f, q * N + i, q);
+        r += ft[q];
+        jx += cx(q) * ft[q];
+        jy += cy(q) * ft[q];
+        jz += cz(q) * ft[q];
+      }
+      // U = sum c f~ - g, u = U + g/2, v = U - g/lambda_-
+      const double Ux = jx - p.g[0], Uy = jy - p.g[1], Uz = jz - p.g[2];
+      const double ux = Ux + 0.5 * p.g[0], uy = Uy + 0.5 * p.g[1], uz = Uz + 0.5 * p.g[2];
+      const double vx = Ux - p.g[0] / p.lam_m, vy = Uy - p.g[1] / p.lam_m, vz = Uz - p.g[2] / p.lam_m;
+      f0[0] = eplus_d(p, 0, r, ux, uy, uz) + (ft[0] - eplus_d(p, 0, r, ux, uy, uz)) / (1.0 + p.lam_p);
+#pragma unroll
+      for (int q = 1; q < 19; q += 2) {
+        const int qb = q + 1;
+        double w = q <= 6 ? 1.0 / 18.0 : 1.0 / 36.0;
+        double ep = eplus_d(p, q, r, ux, uy, uz);
+        double em = 3.0 * w * (cx(q) * vx + cy(q) * vy + cz(q) * vz);
+        double fp = ep + (0.5 * (ft[q] + ft[qb]) - ep) / (1.0 + p.lam_p);
+        double fm = em + (0.5 * (ft[q] - ft[qb]) - em) / (1.0 + p.lam_m);
+        f0[q] = fp + fm;
+        f0[qb] = fp - fm;
       }
     }
     collide_rev(p, f0, ab, fb, th);
@@ -709,44 +938,68 @@ __global__ void __launch_bounds__(128) k_adj_conv1(Par p, const uint8_t* __restr
   const size_t N = (size_t)p.N;
   double th[5] = {0, 0, 0, 0, 0};
   const int n1 = *n1p;
-  for (int li = blockIdx.x * blockDim.x + threadIdx.x; li < n1; li += gridDim.x * blockDim.x) {
-    const long long i = FSL_CK(p, ifc1[li], p.N);
+  const int lane = threadIdx.x & 31, stride = gridDim.x * blockDim.x;
+  // (the same rounds on every lane of a warp)
+  for (int first = (blockIdx.x * blockDim.x + threadIdx.x) & ~31; first < n1; first += stride) {
+    const int li = first + lane;
+    const bool on = li < n1;
+    const long long i = FSL_CK(p, ifc1[on ? li : first], p.N);
     const uint8_t k0 = flags0[i] & KIND;
-    double r = 0.0;
+    double rhat = 0.0;
+    if (on) {
+      double r = 0.0;
 #pragma unroll
-    for (int q = 0; q < 19; ++q) r += ldq_full<P>(f1, q * N + i, q);
-    // phi = m / rho after the step
-    const double pb = phibar[i];
-    const double Mhat = mbar[i] + pb / r;
-    const double rhat = -pb * m1[i] / (r * r);
-    Mh[i] = Mhat;
-    rh[i] = rhat;
-    if (k0 != GAS) continue;
+      for (int q = 0; q < 19; ++q) r += ldq_full<P>(f1, q * N + i, q);
+      // phi = m / rho after the step
+      const double pb = phibar[i];
+      const double Mhat = mbar[i] + pb / r;
+      rhat = -pb * m1[i] / (r * r);
+      Mh[i] = Mhat;
+      rh[i] = rhat;
+    }
     // a new cell from gas: f~ = C(f^eq(rbar, ubar)), means over the fluid
     // neighbours (flags before the step) of their rho = sum f~ and
-    // u = sum c f~ - g/2 (rho_0 = 1)
-    int x, y, z;
-    coords(p, i, x, y, z);
+    // u = sum c f~ - g/2 (rho_0 = 1).  The warp takes its new cells one by one,
+    // a neighbour per lane (a thread with its 18 neighbours in turn was a chain
+    // of 100 us)
+    const bool fresh = on && k0 == GAS;
     double rs = 0.0, us[3] = {0.0, 0.0, 0.0};
     int cnt = 0;
-    for (int l = 1; l < 19; ++l) {
-      const long long yj = nbr(p, x, y, z, cx(l), cy(l), cz(l));
-      if (yj < 0 || !is_fluid(flags0[yj] & KIND)) continue;
-      double ry = 0.0, jx = 0.0, jy = 0.0, jz = 0.0;
+    for (unsigned todo = __ballot_sync(0xffffffffu, fresh); todo; todo &= todo - 1u) {
+      const int o = __ffs(todo) - 1;
+      const long long io = (long long)__shfl_sync(0xffffffffu, (int)i, o);
+      int x, y, z;
+      coords(p, io, x, y, z);
+      double m[4] = {0.0, 0.0, 0.0, 0.0};
+      bool use = false;
+      if (lane >= 1 && lane < 19) {
+        const long long yj = nbr(p, x, y, z, cx(lane), cy(lane), cz(lane));
+        use = yj >= 0 && is_fluid(flags0[yj] & KIND);
+        if (use) {
 #pragma unroll
-      for (int q = 0; q < 19; ++q) {
-        const double v = ldq_full<P>(f1, q * N + yj, q);
-        ry += v;
-        jx += cx(q) * v;
-        jy += cy(q) * v;
-        jz += cz(q) * v;
+          for (int q = 0; q < 19; ++q) {
+            const double v = ldq_full<P>(f1, q * N + yj, q);
+            m[0] += v;
+            if (cx(q)) m[1] += cx(q) * v;
+            if (cy(q)) m[2] += cy(q) * v;
+            if (cz(q)) m[3] += cz(q) * v;
+          }
+#pragma unroll
+          for (int k = 0; k < 3; ++k) m[1 + k] -= 0.5 * p.g[k];
+        }
       }
-      rs += ry;
-      us[0] += jx - 0.5 * p.g[0];
-      us[1] += jy - 0.5 * p.g[1];
-      us[2] += jz - 0.5 * p.g[2];
-      ++cnt;
+#pragma unroll
+      for (int d = 16; d > 0; d >>= 1)
+#pragma unroll
+        for (int k = 0; k < 4; ++k) m[k] += __shfl_xor_sync(0xffffffffu, m[k], d);
+      const int c = __popc(__ballot_sync(0xffffffffu, use));
+      if (lane == o) {
+        rs = m[0];
+        us[0] = m[1]; us[1] = m[2]; us[2] = m[3];
+        cnt = c;
+      }
     }
+    if (!fresh) continue;
     ngb[4 * i] = ngb[4 * i + 1] = ngb[4 * i + 2] = ngb[4 * i + 3] = 0.0;
     if (!cnt) continue;
     const double rbar = rs / cnt, ub0 = us[0] / cnt, ub1 = us[1] / cnt, ub2 = us[2] / cnt;
@@ -805,8 +1058,21 @@ __global__ void __launch_bounds__(128) k_adj_conv2(Par p, const uint8_t* __restr
     const uint8_t k0 = flags0[i] & KIND, k1 = flags1[i] & KIND;
     if (li >= n0 && k0 != LIQ) continue;  // (interface before and after: done from ifc0)
     if (k0 == IFC) phibar[i] = 0.0;
-    int x, y, z;
+    int x, y, z, src[19];
     coords(p, i, x, y, z);
+    pull_sources(p, x, y, z, src);  // (x - c_q; the loops below visit x + c_l as src of the opposite link)
+    // the neighbours' kinds first, so that their loads are in flight together
+    unsigned ifc1m = 0u, newm = 0u;
+#pragma unroll
+    for (int l = 1; l < 19; ++l) {
+      const int j = src[inv(l)];
+      const uint8_t a0 = j < 0 ? (uint8_t)WALL : (uint8_t)(flags0[j] & KIND);
+      const uint8_t a1 = j < 0 ? (uint8_t)WALL : (uint8_t)(flags1[j] & KIND);
+      if (a1 == IFC) {
+        ifc1m |= 1u << l;
+        if (a0 == GAS) newm |= 1u << l;
+      }
+    }
     double add = 0.0, mb = 0.0;
     if (k1 == IFC) add += rh[i];                 // rho after the step = sum f~
     if (k0 == LIQ && k1 == IFC) add += Mh[i];    // new from liquid: m = rho + shares
@@ -818,10 +1084,10 @@ __global__ void __launch_bounds__(128) k_adj_conv2(Par p, const uint8_t* __restr
         // the neighbours that are interface after the step
         double s = 0.0;
         int nr = 0;
+#pragma unroll
         for (int l = 1; l < 19; ++l) {
-          const long long r = nbr(p, x, y, z, cx(l), cy(l), cz(l));
-          if (r < 0 || (flags1[r] & KIND) != IFC) continue;
-          s += Mh[r];
+          if (!((ifc1m >> l) & 1u)) continue;
+          s += Mh[src[inv(l)]];
           ++nr;
         }
         const double exb = nr ? s / nr : 0.0;
@@ -830,9 +1096,10 @@ __global__ void __launch_bounds__(128) k_adj_conv2(Par p, const uint8_t* __restr
       }
     }
     double ng0 = 0.0, ng1 = 0.0, ng2 = 0.0, ng3 = 0.0;  // means of the new cells from gas next to i
+#pragma unroll
     for (int l = 1; l < 19; ++l) {
-      const long long j = nbr(p, x, y, z, cx(l), cy(l), cz(l));
-      if (j < 0 || (flags0[j] & KIND) != GAS || (flags1[j] & KIND) != IFC) continue;
+      if (!((newm >> l) & 1u)) continue;
+      const size_t j = (size_t)src[inv(l)];
       ng0 += ngb[4 * j];
       ng1 += ngb[4 * j + 1];
       ng2 += ngb[4 * j + 2];
@@ -896,7 +1163,7 @@ int adj_objective(fslbm* h, double* J, double* norm) {
   AdjointState* A = h->adj;
   if (cudaMemsetAsync(A->red, 0, 4 * 8, h->st) != cudaSuccess) return 1;
   int blocks = (int)((h->par.N + 255) / 256);
-  if (blocks > 152 * 8) blocks = 152 * 8;
+  if (blocks > ADJ_RED_BLOCKS) blocks = ADJ_RED_BLOCKS;
   k_objective<P><<<blocks, 256, 0, h->st>>>(h->par, h->flags, (const typename Form<P>::S*)cur_f(h),
                                             (const typename Form<P>::R*)cur_phi(h), A->objective, A->red);
   double r[2];

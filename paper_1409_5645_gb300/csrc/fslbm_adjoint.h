@@ -41,7 +41,13 @@ struct AdjointState {
   double fwd_ms = 0.0, adj_ms = 0.0;
   size_t bytes = 0;
   bool ready = false;
+  bool live = false;  // belongs to the handle's current state (a new state ends it, its buffers may stay)
 };
+
+// blocks of the objective's reduction, and the doubles of AdjointState::red:
+// result, count, a block counter, then two partial sums per block
+constexpr int ADJ_RED_BLOCKS = 152 * 2;
+constexpr int ADJ_RED_DOUBLES = 8 + 2 * ADJ_RED_BLOCKS;
 
 namespace fsl {
 

@@ -407,7 +407,7 @@ static int begin_state(fslbm* h, const uint8_t* flags, const double* wall_delta,
                        Staged& sw) {
   const size_t N = (size_t)h->par.N;
   if (!flags) return fail(h, FSLBM_ERR_ARG, "flags is NULL");
-  fslbm_free_adjoint(h);
+  fslbm_end_adjoint(h);
   if (where != FSLBM_HOST && where != FSLBM_DEVICE) return fail(h, FSLBM_ERR_ARG, "bad `where`");
   CK(cudaMemcpyAsync(h->flags, flags, N, where == FSLBM_DEVICE ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice,
                      h->st),

@@ -109,7 +109,7 @@ int run_box(fslbm* h, const int lo[3], const int hi[3], void* buf) {
 template <bool UNPACK>
 int box(fslbm* h, const int lo[3], const int hi[3], void* buf) {
   if (!box_ok(h, lo, hi) || !buf || ((uintptr_t)buf & 15)) return FSLBM_ERR_ARG;
-  if (UNPACK) fslbm_free_adjoint(h);  // a changed state ends a differentiation
+  if (UNPACK) fslbm_end_adjoint(h);  // a changed state ends a differentiation
   switch (h->prec) {
     case FSLBM_F64: return run_box<P64, UNPACK>(h, lo, hi, buf);
     case FSLBM_F32: return run_box<P32, UNPACK>(h, lo, hi, buf);

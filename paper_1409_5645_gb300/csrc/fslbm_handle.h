@@ -12,6 +12,8 @@
 struct AdjointState;
 struct fslbm;
 void fslbm_free_adjoint(fslbm* h);
+// a new state ends a differentiation (fslbm_adjoint.cu): its buffers stay up to a limit
+void fslbm_end_adjoint(fslbm* h);
 
 struct fslbm {
   fslbm_params prm;
