@@ -25,6 +25,7 @@
 // where the device allows it, else as four launches.  The result does not
 // depend on list order.
 #include "fslbm_dev.cuh"
+#include "fslbm_fixed.cuh"
 #include "fslbm_kernels.h"
 
 namespace fsl {
@@ -89,6 +90,41 @@ __device__ __forceinline__ void fill_cell(const Par& p, const View<P>& v, int k)
     push(won, v.nglist, &v.cnt[3], v.cap, (int)j, v.err);
   }
 }
+// The FP64 form's new cell from its neighbours' fixed-point moments (rho, j;
+// lanes with `use`): f^eq of the means, collided; lane q builds population q.
+// Its density and momentum are the means themselves (the weights' sums), as a
+// sum over the lanes would give them back up to rounding.
+__device__ __forceinline__ void newg_fixed(const Par& p, const View<P64>& v, long long j, int q, bool use,
+                                           long long xr, const long long (&xj)[3]) {
+  const unsigned FULL = 0xffffffffu;
+  const int lane = threadIdx.x & 31;
+  // (shifted so that 18 of them stay in range)
+  long long m[4] = {use ? xr >> 5 : 0, use ? xj[0] >> 3 : 0, use ? xj[1] >> 3 : 0, use ? xj[2] >> 3 : 0};
+  const int c = __popc(__ballot_sync(FULL, use));
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+    for (int k = 0; k < 4; ++k) m[k] += __shfl_xor_sync(FULL, m[k], o);
+  const double ic = 1.0 / (double)c;
+  const double rho = double_of_fix(m[0]) * 32.0 * ic;
+  const double u0 = double_of_fix(m[1]) * 8.0 * ic - 0.5 * p.g[0], u1 = double_of_fix(m[2]) * 8.0 * ic - 0.5 * p.g[1],
+               u2 = double_of_fix(m[3]) * 8.0 * ic - 0.5 * p.g[2];
+  const double w = q == 0 ? 1.0 / 3.0 : (q <= 6 ? 1.0 / 18.0 : 1.0 / 36.0);
+  const double ax = cx(q), ay = cy(q), az = cz(q);
+  const double cu = ax * u0 + ay * u1 + az * u2, usq = u0 * u0 + u1 * u1 + u2 * u2;
+  const double fp = w * (rho + 1.5 * (3.0 * cu * cu - usq)), fm = 3.0 * w * cu;  // even and odd part of f^eq
+  // the collision moves them toward e^+(u + g/2) and e^-(u - g/lambda_-)
+  const double cg = ax * p.g[0] + ay * p.g[1] + az * p.g[2];
+  const double ug = u0 * p.g[0] + u1 * p.g[1] + u2 * p.g[2], gg = p.g[0] * p.g[0] + p.g[1] * p.g[1] + p.g[2] * p.g[2];
+  const double np = w * 1.5 * ((ug + 0.25 * gg) - 3.0 * cg * (cu + 0.25 * cg));  // f^+ - e^+
+  const double nm = 3.0 * w * cg * p.inv_lam_m;                                   // f^- - e^-
+  if (lane < 19) v.fout[(size_t)q * (size_t)p.N + (size_t)j] = (fp + p.lam_p * np) + (fm + p.lam_m * nm);
+  if (lane == 0) {
+    v.m[j] = 0.0;
+    v.phout[j] = 0.0;
+  }
+}
+
 // new cell k by a warp: lane l (1..18) reads neighbour l's populations; the
 // means are summed in neighbour order; lane q builds and collides population q
 template <int P>
@@ -102,8 +138,9 @@ __device__ __forceinline__ void newg_cell(const Par& p, const View<P>& v, int k)
     const long long j = FSL_CK(p, v.nglist[k], p.N);
     int x, y, z;
     coords(p, j, x, y, z);
-    bool use = false;
+    bool use = false, range = true;
     R rr = R(0), ux = R(0), uy = R(0), uz = R(0);
+    long long xr = 0, xj[3] = {0, 0, 0};  // the neighbour's moments in fixed point (FP64 form)
     if (lane >= 1 && lane < 19) {
       long long y2 = nbr(p, x, y, z, cx(q), cy(q), cz(q));
       if (y2 >= 0) {
@@ -112,7 +149,28 @@ __device__ __forceinline__ void newg_cell(const Par& p, const View<P>& v, int k)
 #pragma unroll
         for (int r = 0; r < 19; ++r) g[r] = ldq<P>(v.fout, (size_t)r * N + (size_t)y2, r);
         use = is_fluid(v.flags[y2] & KIND);
-        if (use) moments_post<R, Form<P>::SH>(p, g, rr, ux, uy, uz);
+        if (use) {
+          if constexpr (P == P64) {
+            range = p.fix_ok && moments_fixed(g, xr, xj);
+            if (!range) moments_post<R, Form<P>::SH>(p, g, rr, ux, uy, uz);
+          } else {
+            moments_post<R, Form<P>::SH>(p, g, rr, ux, uy, uz);
+          }
+        }
+      }
+    }
+    if constexpr (P == P64) {
+      // every neighbour in range: the sums are exact in any order, and the FP64
+      // pipe (which bounded the stage) sees four conversions
+      if (__all_sync(FULL, range)) {
+        newg_fixed(p, v, j, q, use, xr, xj);
+        return;
+      }
+      if (use && range) {
+        rr = double_of_fix(xr);
+        ux = double_of_fix(xj[0]) - 0.5 * p.g[0];
+        uy = double_of_fix(xj[1]) - 0.5 * p.g[1];
+        uz = double_of_fix(xj[2]) - 0.5 * p.g[2];
       }
     }
     R rs = R(0), s0 = R(0), s1 = R(0), s2 = R(0);
@@ -205,12 +263,29 @@ __device__ __forceinline__ void empty_cell(const Par& p, const View<P>& v, int k
   }
 }
 
+// The calling warp's place among the grid's: the blocks' first warps, then their
+// second ones, ..., so that a list shorter than the grid spreads over every SM
+// (by blocks, 900 items of a 128x64x64 splash sat on a third of the SMs and
+// its 5 k receivers, a thread each, on ten).
+__device__ __forceinline__ int grid_warp() { return (int)((threadIdx.x >> 5) * gridDim.x + blockIdx.x); }
+__device__ __forceinline__ int grid_warps() { return (int)((blockDim.x >> 5) * gridDim.x); }
+// items of a thread each: few lanes of every warp where the list is short
+struct LaneItems {
+  int k, step, end;
+  __device__ __forceinline__ explicit LaneItems(int n, int first_warp) {
+    const int nw = grid_warps(), lane = threadIdx.x & 31;
+    const int per = min(max((n + nw - 1) / nw, 1), 32);  // items per warp and round
+    k = lane < per ? first_warp * per + lane : n;
+    step = nw * per;
+    end = n;
+  }
+};
+
 // the first stage: a warp per fill or empty cell
 template <int P>
 __device__ __forceinline__ void do_fill_empty(const Par& p, const View<P>& v) {
   const int nf = min(load_count(&v.cnt[1]), v.cap), ne = min(load_count(&v.cnt[2]), v.cap);
-  const int nw = (gridDim.x * blockDim.x) >> 5;
-  for (int k = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; k < nf + ne; k += nw) {
+  for (int k = grid_warp(); k < nf + ne; k += grid_warps()) {
     if (k < nf) fill_cell<P>(p, v, k);
     else empty_cell<P>(p, v, k - nf);
   }
@@ -222,14 +297,13 @@ __global__ void __launch_bounds__(256) k_fill_empty(Par p, View<P> v) {
 }
 
 // liquid cells turned interface next to an emptied cell: m = rho, phi = m/rho
-// (by the grid's last threads first: its first warps take the other items of
-// the stage)
+// (by the grid's last warps first: its first ones take the other items of the
+// stage)
 template <int P>
 __device__ __forceinline__ void do_newl(const Par& p, const View<P>& v) {
   using R = typename Form<P>::R;
-  int nl = min(load_count(&v.cnt[4]), v.cap);
-  const int nt = gridDim.x * blockDim.x;
-  for (int k = nt - 1 - (int)(blockIdx.x * blockDim.x + threadIdx.x); k < nl; k += nt) {
+  const LaneItems it(min(load_count(&v.cnt[4]), v.cap), grid_warps() - 1 - grid_warp());
+  for (int k = it.k; k < it.end; k += it.step) {
     long long j = FSL_CK(p, v.nllist[k], p.N);
     const double r = rho_out<P>(p, v, j);
     v.m[j] = r;
@@ -337,8 +411,7 @@ template <int P>
 __device__ __forceinline__ void do_new_share(const Par& p, const View<P>& v) {
   const int nf = min(load_count(&v.cnt[1]), v.cap), ne = min(load_count(&v.cnt[2]), v.cap);
   const int nn = min(load_count(&v.cnt[3]), v.cap);
-  const int nw = (gridDim.x * blockDim.x) >> 5;
-  for (int k = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; k < nn + nf + ne; k += nw) {
+  for (int k = grid_warp(); k < nn + nf + ne; k += grid_warps()) {
     if (k < nn) newg_cell<P>(p, v, k);
     else share_cell<P>(p, v, k - nn, nf);
   }
@@ -355,9 +428,9 @@ __global__ void __launch_bounds__(256) k_new_share(Par p, View<P> v) {
 template <int P>
 __device__ __forceinline__ void do_recv(const Par& p, const View<P>& v) {
   using R = typename Form<P>::R;
-  const int nr = min(load_count(&v.cnt[5]), v.cap);
+  const LaneItems it(min(load_count(&v.cnt[5]), v.cap), grid_warp());
   const long long sy = p.nx, sz = (long long)p.nx * p.ny;
-  for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < nr; k += gridDim.x * blockDim.x) {
+  for (int k = it.k; k < it.end; k += it.step) {
     const long long yj = FSL_CK(p, v.rlist[k], p.N);
     int x, y, z;
     coords(p, yj, x, y, z);
@@ -425,7 +498,8 @@ __device__ __forceinline__ void do_final(const Par& p, const View<P>& v) {
   // running total of conversions since the state was set (never reset per step)
   if (blockIdx.x == 0 && threadIdx.x == 0 && nf + ng + nl) atomicAdd(&v.cnt[8], nf + ng + nl);
   int emptied = 0;  // cells this thread turned to gas (counted once per warp below)
-  for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < total; k += gridDim.x * blockDim.x) {
+  const LaneItems it(total, grid_warp());
+  for (int k = it.k; k < it.end; k += it.step) {
     int kk = k;
     if (kk < nf) {
       long long i = FSL_CK(p, v.flist[kk], p.N);
@@ -486,11 +560,15 @@ __global__ void __launch_bounds__(256) k_final(Par p, View<P> v) {
 // counter cnt[10] and waits until the blocks of this phase have arrived.  The
 // wait is bounded (about a second); on expiry it records ERRB_SYNC and goes
 // on, the step's result is then invalid and the host reports the error.
-__device__ __forceinline__ void grid_sync(unsigned* ctr, unsigned target, int* err) {
+__device__ __forceinline__ void grid_arrive(unsigned* ctr) {
   __syncthreads();
   if (threadIdx.x == 0) {
     __threadfence();
     atomicAdd(ctr, 1u);
+  }
+}
+__device__ __forceinline__ void grid_wait(unsigned* ctr, unsigned target, int* err) {
+  if (threadIdx.x == 0) {
     unsigned spins = 0;
     while (*((volatile unsigned*)ctr) < target) {
       if (++spins > (1u << 20)) {
@@ -504,39 +582,55 @@ __device__ __forceinline__ void grid_sync(unsigned* ctr, unsigned target, int* e
   __syncthreads();
 }
 
-// the four conversion stages in one launch, separated by grid barriers; the
-// step's two-level mass reduction (the same chunks and order as the
-// stand-alone pair of launches) is carried by the grid's last blocks, the
-// last of them to finish its chunk adding up the chunks: it reads the lost
-// ledger before its block arrives at the first barrier, so before any excess
-// of this step reaches it.  A step without a fill or an empty cell ends there
-// (alone, with warm caches: a film's step 17.2 -> 6.8 us; with conversions, the
-// items of a stage spread over the warps and the receivers' loads together,
-// a 128x64x64 splash's 46.8 -> 35.0 us)
+__device__ __forceinline__ void grid_sync(unsigned* ctr, unsigned target, int* err) {
+  grid_arrive(ctr);
+  grid_wait(ctr, target, err);
+}
+
+// The step's two-level mass reduction (the same chunks and order as the
+// stand-alone pair of launches) on the grid's last blocks: a chunk each, and
+// the last of them to finish adds up the chunks.  lost0: the lost ledger before
+// any excess of this step (thread 0).
+__device__ __forceinline__ void reduce_mass(const MassReduce& mr, int chunk, int* done, double lost0) {
+  if (chunk < 0) return;  // (block-uniform)
+  __shared__ bool last;
+  const double t = block_chunk_sum(mr.in, mr.n, mr.chunk, chunk);
+  if (threadIdx.x == 0) {
+    mr.tmp[chunk] = t;
+    __threadfence();
+    last = atomicAdd(done, 1) == mr.nb - 1;
+    __threadfence();
+  }
+  __syncthreads();
+  if (last) {
+    const double m = block_chunk_sum<true>(mr.tmp, mr.nb, mr.nb, 0);
+    if (threadIdx.x == 0) *mr.out = m + lost0;
+  }
+}
+
+// the four conversion stages in one launch, separated by grid barriers, with
+// the mass reduction between a block's arrival at the first barrier and its
+// wait there.  A step without a fill or an empty cell has the mass only.
+// Alone, with warm caches: a film's step 17.2 -> 6.8 us without the barriers;
+// with conversions, a stage's items one to a warp over all SMs and a
+// receiver's loads together, a 128x64x64 splash's 46.8 -> 38.8 us, a 256x128x128 FP64
+// splash's 96 -> 60 us
 template <int P>
 __global__ void __launch_bounds__(256) k_convert(Par p, View<P> v, MassReduce mr) {
   pdl_begin();
   unsigned* ctr = (unsigned*)&v.cnt[10];
   const unsigned nb = gridDim.x;
   const int chunk = (int)blockIdx.x - ((int)gridDim.x - mr.nb);
-  if (chunk >= 0) {
-    __shared__ bool last;
-    const double t = block_chunk_sum(mr.in, mr.n, mr.chunk, chunk);
-    if (threadIdx.x == 0) {
-      mr.tmp[chunk] = t;
-      __threadfence();
-      last = atomicAdd(&v.cnt[11], 1) == mr.nb - 1;
-      __threadfence();
-    }
-    __syncthreads();
-    if (last) {
-      const double m = block_chunk_sum<true>(mr.tmp, mr.nb, mr.nb, 0);
-      if (threadIdx.x == 0) *mr.out = m + *mr.add;
-    }
+  double lost0 = 0.0;
+  if (chunk >= 0 && threadIdx.x == 0) lost0 = *((volatile const double*)mr.add);
+  if (load_count(&v.cnt[1]) + load_count(&v.cnt[2]) == 0) {  // (settled before this kernel)
+    reduce_mass(mr, chunk, &v.cnt[11], lost0);
+    return;
   }
-  if (load_count(&v.cnt[1]) + load_count(&v.cnt[2]) == 0) return;  // (settled before this kernel)
   do_fill_empty<P>(p, v);
-  grid_sync(ctr, nb, v.err);
+  grid_arrive(ctr);
+  reduce_mass(mr, chunk, &v.cnt[11], lost0);
+  grid_wait(ctr, nb, v.err);
   do_new_share<P>(p, v);
   grid_sync(ctr, 2 * nb, v.err);
   do_recv<P>(p, v);

@@ -165,4 +165,90 @@ __host__ __device__ __forceinline__ bool collide_fixed(const Par& p, double (&f)
   return true;
 }
 
+#ifdef __CUDACC__
+// collide_fixed with population q on lane q of a warp (q = 0 on the lanes from
+// 19 on): the same integers, so the same bits.  False, with f untouched, where
+// the cell is out of range.
+__device__ __forceinline__ bool collide_warp(const Par& p, int q, double& f, long long& rho) {
+  const unsigned FULL = 0xffffffffu;
+  if (!p.fix_ok) return false;
+  const int lane = threadIdx.x & 31, qb = q == 0 ? 0 : ((q & 1) ? q + 1 : q - 1);
+  const unsigned h = (unsigned)(bits_of_double(f) >> 32);
+  bool ok = __all_sync(FULL, h < (q ? 0x3fd00000u : 0x3ff00000u));
+  const long long x = ok ? fix_of(bits_of_double(f)) : 0;
+  long long m[4] = {0, 0, 0, 0};
+  if (lane < 19) {
+    m[0] = x;
+    m[1] = cx(q) * x;
+    m[2] = cy(q) * x;
+    m[3] = cz(q) * x;
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+    for (int k = 0; k < 4; ++k) m[k] += __shfl_xor_sync(FULL, m[k], o);
+  auto half = [](long long j) { return (unsigned)((int)(j >> 32) + 0x08000000) < 0x10000000u; };
+  ok = ok && half(m[1]) && half(m[2]) && half(m[3]);  // (the same on every lane)
+  if (!ok) return false;
+  const long long ux = (m[1] + p.fx_hg[0]) << 2, uy = (m[2] + p.fx_hg[1]) << 2, uz = (m[3] + p.fx_hg[2]) << 2;
+  const long long xx = mul_hi_near(ux, ux), yy = mul_hi_near(uy, uy), zz = mul_hi_near(uz, uz);
+  const long long xy = mul_hi_near(ux, uy), xz = mul_hi_near(ux, uz), yz = mul_hi_near(uy, uz);
+  const long long usq = xx + yy + zz, dens = m[0] - usq - (usq >> 1);
+  constexpr long long K36 = 0x071c71c71c71c700LL, K3 = 0x5555555555555400LL, K12 = 0x1555555555555500LL;
+  const long long a = mul_hi_near(dens, K36);
+  const long long bx = mul_hi_near(m[1] - p.fx_gl[0], K12), by = mul_hi_near(m[2] - p.fx_gl[1], K12),
+                  bz = mul_hi_near(m[3] - p.fx_gl[2], K12);
+  const long long xb = __shfl_sync(FULL, x, qb);
+  long long y;
+  if (q == 0) {
+    y = x + mul_hi_near(p.fx_lp, (x - mul_hi_near(dens, K3)) << 2);
+  } else {
+    // the odd link's terms, as collide_fixed takes them, on both lanes of a pair
+    const int qo = (q & 1) ? q : qb;
+    long long e2, m2;
+    if (qo <= 6) {
+      e2 = 4 * a + ((qo == 1 ? xx : (qo == 3 ? yy : zz)) >> 1);
+      m2 = 4 * (qo == 1 ? bx : (qo == 3 ? by : bz));
+    } else {
+      const long long s = qo <= 10 ? xx + yy : (qo <= 14 ? xx + zz : yy + zz);
+      const long long c = qo <= 10 ? xy : (qo <= 14 ? xz : yz);
+      const int cxo = cx(qo), cyo = cy(qo), czo = cz(qo);
+      const bool same = cxo * cyo + cxo * czo + cyo * czo > 0;
+      e2 = 2 * a + ((same ? s + 2 * c : s - 2 * c) >> 2);
+      m2 = 2 * (cxo * bx + cyo * by + czo * bz);
+    }
+    const long long d = (q & 1) ? x - xb : xb - x;
+    const long long rp = mul_hi_near(p.fx_lp, (x + xb - e2) << 1), rm = mul_hi_near(p.fx_lm, (d - m2) << 1);
+    y = x + rp + ((q & 1) ? rm : -rm);
+  }
+  // (both conversions round the same; a thread chooses one for its 19)
+  f = y >= (1LL << 32) ? double_of_bits(bits_of(y)) : double_of_fix(y);
+  rho = m[0];
+  return true;
+}
+#endif
+
+// density and momentum of populations in the collision's range, in units of
+// 2^-60; false where they are not
+__host__ __device__ __forceinline__ bool moments_fixed(const double (&f)[19], long long& rho, long long (&j)[3]) {
+  unsigned top = 0u;
+#pragma unroll
+  for (int q = 1; q < 19; ++q) {
+    const unsigned h = (unsigned)(bits_of_double(f[q]) >> 32);
+    top = h > top ? h : top;
+  }
+  if (!(top < 0x3fd00000u && (unsigned)(bits_of_double(f[0]) >> 32) < 0x3ff00000u)) return false;
+  rho = fix_of(bits_of_double(f[0]));
+  j[0] = j[1] = j[2] = 0;
+#pragma unroll
+  for (int q = 1; q < 19; q += 2) {
+    const long long a = fix_of(bits_of_double(f[q])), b = fix_of(bits_of_double(f[q + 1]));
+    rho += a + b;
+    j[0] += cx(q) * (a - b);
+    j[1] += cy(q) * (a - b);
+    j[2] += cz(q) * (a - b);
+  }
+  return true;
+}
+
 }  // namespace fsl

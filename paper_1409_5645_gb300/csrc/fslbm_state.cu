@@ -136,8 +136,9 @@ __global__ void k_prepare_flags(Par p, uint8_t* flags, int* err) {
 // The same with 16 cells of a row per thread (nx a multiple of 16): the kinds
 // are one-hot, so the OR of the neighbours' bytes holds their kinds; nine
 // 16-byte loads and ten single bytes instead of 18 bytes a cell (512x256x256:
-// 953 -> 96 us).  Cells on the y and z faces, and a row's
-// first and last group on a periodic x axis, take the cell path.  The bits written beside
+// 953 -> 90 us; its faces cell by cell took longer than the rest
+// of a small lattice).  A row's first and last group on a periodic
+// x axis take the cell path.  The bits written beside
 // the kinds are masked from every load, so cells may be rewritten while their
 // neighbours read them.
 __global__ void __launch_bounds__(256) k_prepare_flags16(Par p, uint8_t* flags, int* err) {
@@ -149,16 +150,24 @@ __global__ void __launch_bounds__(256) k_prepare_flags16(Par p, uint8_t* flags, 
     int x, y, z;
     coords(p, i, x, y, z);
     const bool xlo = x == 0, xhi = x + 16 == p.nx;
-    if (((xlo || xhi) && p.px) || y == 0 || y == p.ny - 1 || z == 0 || z == p.nz - 1) {
+    if ((xlo || xhi) && p.px) {
       for (int k = 0; k < 16; ++k) prepare_cell(p, flags, err, i + k, x + k, y, z);
       continue;
     }
     unsigned near[4] = {0u, 0u, 0u, 0u}, own[4] = {0u, 0u, 0u, 0u};
+    bool face = false;  // a row of neighbours lies past a non-periodic face
 #pragma unroll
     for (int dz = -1; dz <= 1; ++dz)
 #pragma unroll
       for (int dy = -1; dy <= 1; ++dy) {
-        const uint8_t* row = flags + (i + dy * sy + dz * sz);
+        int Y = y + dy, Z = z + dz;
+        if (p.py) Y += Y < 0 ? p.ny : (Y >= p.ny ? -p.ny : 0);
+        if (p.pz) Z += Z < 0 ? p.nz : (Z >= p.nz ? -p.nz : 0);
+        if ((unsigned)Y >= (unsigned)p.ny || (unsigned)Z >= (unsigned)p.nz) {
+          face = true;
+          continue;
+        }
+        const uint8_t* row = flags + (x + sy * Y + sz * Z);
         const uint4 w4 = *reinterpret_cast<const uint4*>(row);
         const unsigned w[4] = {w4.x, w4.y, w4.z, w4.w};
         const bool centre = dy == 0 && dz == 0;
@@ -189,7 +198,7 @@ __global__ void __launch_bounds__(256) k_prepare_flags16(Par p, uint8_t* flags, 
       bad = bad || b0 + b1 + b2 + b3 != one;                  // each byte one kind (no carry: at most 4)
       bad = bad || (b0 & ((near[k] >> 2) & one)) != 0u;       // a liquid cell next to gas
       const unsigned wall = (near[k] >> 3) & one;
-      o[k] = own[k] | (wall * (unsigned)(NEARB | NEARW));
+      o[k] = own[k] | (wall * (unsigned)(NEARB | NEARW)) | (face ? one * (unsigned)NEARB : 0u);
     }
     if (xlo) o[0] |= NEARB;  // (beyond a non-periodic face: a wall)
     if (xhi) o[3] |= (unsigned)NEARB << 24;
