@@ -304,22 +304,98 @@ __device__ __forceinline__ double iface_cell(const Par& p, const View<P>& v, int
   return mm;
 }
 
-// c_q . a for an unrolled q
-template <class R>
-__device__ __forceinline__ R cdot(int q, const R (&a)[3]) {
-  R s = R(0);
-  if (cx(q)) s = cx(q) > 0 ? a[0] : -a[0];
-  if (cy(q)) s = cx(q) ? (cy(q) > 0 ? s + a[1] : s - a[1]) : (cy(q) > 0 ? a[1] : -a[1]);
-  if (cz(q)) s = (cx(q) || cy(q)) ? (cz(q) > 0 ? s + a[2] : s - a[2]) : (cz(q) > 0 ? a[2] : -a[2]);
-  return s;
-}
-
 // The FP64 form's default interface cell.  Its FP64 pipe (two operations a
 // cycle and SM) bounds it, so the arithmetic is laid out for few of them: the
 // equilibria, the non-equilibrium part and the quotient d / (n.c) are taken
 // once per link pair (a pair has at most one link with the FSL closure: its
 // upstream node must be fluid), both directions of a pair run the same
 // instructions on selected operands, and the collision is the fixed-point one.
+// It comes for a thread per cell and, where the list is short, for a warp per
+// cell with a link per lane; every rounding is written out, so the two give
+// the same bits and the choice does not show.
+//
+// c . a for a link with components 0 or +-1 (one rounding, of the sum)
+__device__ __forceinline__ double link_dot(int ax, int ay, int az, const double (&a)[3]) {
+  return fx_fma((double)ax, a[0], fx_fma((double)ay, a[1], fx_mul((double)az, a[2])));
+}
+
+// what the links of a cell share
+struct Surface64 {
+  double n[3], d;        // the plane of k_geom
+  double rb, rt;         // rho_b and rho(t)
+  double r0b, r0t;       // rho_0 beside them
+  double u[3], usq, nl;  // u_b, its square, 0 for the linear equilibrium
+};
+
+// The closure of the pair of links q (components a) and its opposite qb:
+// o / ob the cell's own populations, f / fb the pulled ones, ga / gb whether
+// they come from gas, blocked whether from gas or a wall; w the weight.
+// Rebuilds f and fb.
+__device__ __forceinline__ void gas_pair64(const Par& p, const Surface64& S, double w, int ax, int ay, int az, double o,
+                                           double ob, bool ga, bool gb, bool ba, bool bb, double& f, double& fb) {
+  // e^+ of both directions: w rho + 3/2 w rho_0 (3 (c.u)^2 - u.u)
+  const double cu = link_dot(ax, ay, az, S.u);
+  const double k = fx_mul(fx_mul(S.nl, fx_mul(1.5, w)), fx_fma(fx_mul(3.0, cu), cu, -S.usq));
+  const double eb = fx_fma(S.r0b, k, fx_mul(w, S.rb));
+  // FSL (Table 1): the rebuilt population's own link has a fluid upstream node
+  const bool fa = p.rule != 0 && ga && !bb, fo = p.rule != 0 && gb && !ba;
+  double val = 0.0;
+  if (fa || fo) {
+    const double hs = fx_mul(0.5, fx_add(o, ob));
+    const double nplus = fx_mul(fx_sub(hs, fx_fma(S.r0t, k, fx_mul(w, S.rt))), p.inv_1plp);
+    const double op = fa ? ob : o, fup = fa ? fb : f;
+    const double cq = link_dot(ax, ay, az, S.n), cn = fa ? -cq : cq;
+    double dl = 0.5;
+    if (cn > 0.0) {
+      dl = __ddiv_rn(S.d, cn);
+      dl = dl < p.delta_min ? p.delta_min : (dl > 1.0 ? 1.0 : dl);
+    }
+    val = fx_add(fx_add(fx_sub(hs, fup), eb), fx_fma(dl, fx_sub(fup, op), fx_mul(fx_mul(p.lam_p, fx_sub(dl, 1.5)), nplus)));
+  }
+  const double ska = fx_fma(2.0, eb, -ob), skb = fx_fma(2.0, eb, -o);  // FSK, Eq. koerner
+  if (ga) f = fa ? val : ska;
+  if (gb) fb = fo ? val : skb;
+}
+
+// plane, densities and velocity of a cell from its geometry and the moments of
+// its own populations
+__device__ __forceinline__ void surface64(const Par& p, const View<P64>& v, int li, double rt, const double (&j)[3],
+                                          Surface64& S) {
+  S.n[0] = S.n[1] = S.n[2] = S.d = 0.0;
+  S.rb = p.rho_G;
+  if (p.rule != 0 || p.sigma != 0.0) {
+    const size_t cap = (size_t)v.cap;
+    S.n[0] = v.geo[li];
+    S.n[1] = v.geo[cap + li];
+    S.n[2] = v.geo[2 * cap + li];
+    S.d = v.geo[3 * cap + li];
+    S.rb = fx_fma(fx_mul(3.0, p.sigma), v.geo[4 * cap + li], S.rb);
+  }
+  S.rt = rt;
+  S.r0t = p.compressible ? rt : 1.0;
+  S.r0b = p.compressible ? S.rb : 1.0;
+#pragma unroll
+  for (int a = 0; a < 3; ++a) S.u[a] = fx_fma(-0.5, p.g[a], p.compressible ? __ddiv_rn(j[a], rt) : j[a]);
+  S.usq = fx_fma(S.u[2], S.u[2], fx_fma(S.u[1], S.u[1], fx_mul(S.u[0], S.u[0])));
+  S.nl = p.linear_eq ? 0.0 : 1.0;
+}
+
+// the cell's new mass and fill level and its conversion marks (one thread)
+__device__ __forceinline__ double finish64(const Par& p, const View<P64>& v, long long i, double dm, double rho,
+                                           unsigned wallm, unsigned gasm, bool& fill, bool& empty) {
+  double mm = v.m[i];
+  if (!p.freeze) {
+    mm = fx_add(mm, dm);
+    v.m[i] = mm;
+    v.phout[i] = __ddiv_rn(mm, rho);
+    fill = mm > fx_mul(1.0 + p.eps, rho) || ((p.cleanup & 1) && gasm == 0u);
+    empty = !fill && (mm < fx_mul(-p.eps, rho) || ((p.cleanup & 2) && (wallm | gasm) == 0x7fffeu));
+    if (fill) v.mark[i] = MK_FILL;
+    else if (empty) v.mark[i] = MK_EMPTY;
+  }
+  return mm;
+}
+
 template <bool IN>
 __device__ __forceinline__ double iface_cell64(const Par& p, const View<P64>& v, int li, long long i, int x, int y,
                                                int z, bool& fill, bool& empty) {
@@ -341,64 +417,31 @@ __device__ __forceinline__ double iface_cell64(const Par& p, const View<P64>& v,
       if ((wallm | gasm) & (1u << q)) continue;
       const long long sq = IN ? FSL_CK(p, i - (cx(q) + sy * cy(q) + sz * cz(q)), p.N) : (long long)srcs[q];
       const double phs = v.phin[sq];
-      dm += ((liqm & (1u << q)) ? 2.0 : phic + phs) * (f[q] - own[inv(q)]);
+      dm = fx_fma((liqm & (1u << q)) ? 2.0 : fx_add(phic, phs), fx_sub(f[q], own[inv(q)]), dm);
     }
-    dm *= 0.5;
+    dm = fx_mul(0.5, dm);
   }
   if (wallm) wall_links<P64>(p, v, i, wallm, gasm, own, f);
   if (gasm) {
-    double n[3] = {0.0, 0.0, 0.0}, d = 0.0, rb = p.rho_G;
-    if (p.rule != 0 || p.sigma != 0.0) {
-      const size_t cap = (size_t)v.cap;
-      n[0] = v.geo[li];
-      n[1] = v.geo[cap + li];
-      n[2] = v.geo[2 * cap + li];
-      d = v.geo[3 * cap + li];
-      rb += 3.0 * p.sigma * v.geo[4 * cap + li];
-    }
     double rt = own[0], j[3] = {0.0, 0.0, 0.0};
 #pragma unroll
     for (int q = 1; q < 19; q += 2) {
-      const double s = own[q] + own[q + 1], e = own[q] - own[q + 1];
-      rt += s;
-      if (cx(q)) j[0] += cx(q) * e;
-      if (cy(q)) j[1] += cy(q) * e;
-      if (cz(q)) j[2] += cz(q) * e;
+      const double s = fx_add(own[q], own[q + 1]), e = fx_sub(own[q], own[q + 1]);
+      rt = fx_add(rt, s);
+      if (cx(q)) j[0] = fx_add(j[0], cx(q) * e);
+      if (cy(q)) j[1] = fx_add(j[1], cy(q) * e);
+      if (cz(q)) j[2] = fx_add(j[2], cz(q) * e);
     }
-    const double r0t = p.compressible ? rt : 1.0, r0b = p.compressible ? rb : 1.0;
-    double u[3];
-#pragma unroll
-    for (int a = 0; a < 3; ++a) u[a] = (p.compressible ? j[a] / rt : j[a]) - 0.5 * p.g[a];
-    const double usq = u[0] * u[0] + u[1] * u[1] + u[2] * u[2], nl = p.linear_eq ? 0.0 : 1.0;
+    Surface64 S;
+    surface64(p, v, li, rt, j, S);
+    const unsigned blocked = wallm | gasm;
 #pragma unroll
     for (int q = 1; q < 19; q += 2) {
-      constexpr double w1 = 1.0 / 18.0, w7 = 1.0 / 36.0;
-      const double w = q <= 6 ? w1 : w7;
       const int qb = q + 1;
       const bool ga = (gasm >> q) & 1u, gb = (gasm >> qb) & 1u;
-      if (!(ga || gb)) continue;
-      // e^+ of both directions: w rho + 3/2 w rho_0 (3 (c.u)^2 - u.u)
-      const double cu = cdot<double>(q, u), k = nl * (4.5 * w * cu * cu - 1.5 * w * usq);
-      const double eb = w * rb + r0b * k;
-      const unsigned blocked = wallm | gasm;
-      // FSL (Table 1): the rebuilt population's own link (q from qb's gas) has a fluid upstream node
-      const bool fa = p.rule != 0 && ga && !((blocked >> qb) & 1u), fb = p.rule != 0 && gb && !((blocked >> q) & 1u);
-      double val = 0.0;
-      if (fa || fb) {
-        const double s = own[q] + own[qb];
-        const double nplus = (0.5 * s - (w * rt + r0t * k)) * p.inv_1plp;
-        const double op = fa ? own[qb] : own[q], fup = fa ? f[qb] : f[q];
-        const double cq = cdot<double>(q, n), cn = fa ? -cq : cq;
-        double dl = 0.5;
-        if (cn > 0.0) {
-          dl = d / cn;
-          dl = dl < p.delta_min ? p.delta_min : (dl > 1.0 ? 1.0 : dl);
-        }
-        val = 0.5 * s - fup + dl * (fup - op) + p.lam_p * (dl - 1.5) * nplus + eb;
-      }
-      const double ska = 2.0 * eb - own[qb], skb = 2.0 * eb - own[q];  // FSK, Eq. koerner
-      if (ga) f[q] = fa ? val : ska;
-      if (gb) f[qb] = fb ? val : skb;
+      if (ga || gb)
+        gas_pair64(p, S, q <= 6 ? 1.0 / 18.0 : 1.0 / 36.0, cx(q), cy(q), cz(q), own[q], own[qb], ga, gb,
+                   (blocked >> q) & 1u, (blocked >> qb) & 1u, f[q], f[qb]);
     }
   }
   double rho;
@@ -413,17 +456,91 @@ __device__ __forceinline__ double iface_cell64(const Par& p, const View<P64>& v,
   }
 #pragma unroll
   for (int q = 0; q < 19; ++q) v.fout[(size_t)q * N + (size_t)i] = f[q];
-  double mm = v.m[i];
+  return finish64(p, v, i, dm, rho, wallm, gasm, fill, empty);
+}
+
+// A cell by a warp, link q on lane q (the lanes from 19 on repeat the rest
+// population and write nothing); fill, empty and the returned mass are lane 0's.
+__device__ __forceinline__ double iface_warp64(const Par& p, const View<P64>& v, int li, long long i, int x, int y,
+                                               int z, bool& fill, bool& empty) {
+  const unsigned FULL = 0xffffffffu;
+  const size_t N = (size_t)p.N;
+  const int lane = threadIdx.x & 31, q = lane < 19 ? lane : 0, qb = q == 0 ? 0 : ((q & 1) ? q + 1 : q - 1);
+  const int ax = cx(q), ay = cy(q), az = cz(q);
+  const long long s = nbr(p, x, y, z, -ax, -ay, -az);
+  const uint8_t ks = kind_at(v.flags, s);
+  const double own = v.fin[(size_t)q * N + (size_t)i];
+  double f = v.fin[(size_t)q * N + (size_t)(s < 0 ? 0 : s)];
+  const double phic = v.phin[i], phs = s < 0 ? 0.0 : v.phin[s];
+  if (!is_fluid(ks)) f = 0.0;
+  const bool link = lane >= 1 && lane < 19;
+  const unsigned wallm = __ballot_sync(FULL, link && ks == WALL);
+  const unsigned gasm = __ballot_sync(FULL, link && ks != WALL && !is_fluid(ks));
+  const unsigned blocked = wallm | gasm;
+  const double ownb = __shfl_sync(FULL, own, qb);
+  double dm = 0.0;
   if (!p.freeze) {
-    mm = mm + dm;
-    v.m[i] = mm;
-    v.phout[i] = mm / rho;
-    fill = mm > (1.0 + p.eps) * rho || ((p.cleanup & 1) && gasm == 0u);
-    empty = !fill && (mm < -p.eps * rho || ((p.cleanup & 2) && (wallm | gasm) == 0x7fffeu));
-    if (fill) v.mark[i] = MK_FILL;
-    else if (empty) v.mark[i] = MK_EMPTY;
+    const double wgt = ks == LIQ ? 2.0 : fx_add(phic, phs), dif = fx_sub(f, ownb);
+#pragma unroll
+    for (int l = 1; l < 19; ++l) {  // in link order, as a thread sums it
+      const double a = __shfl_sync(FULL, wgt, l), b = __shfl_sync(FULL, dif, l);
+      if (!((blocked >> l) & 1u)) dm = fx_fma(a, b, dm);
+    }
+    dm = fx_mul(0.5, dm);
   }
-  return mm;
+  double fb = __shfl_sync(FULL, f, qb);  // the opposite link's pulled value
+  if ((wallm >> q) & 1u) {  // (wall_links)
+    double val = ownb;
+    if (p.has_wd) {
+      const double dw = v.wd[(size_t)qb * N + (size_t)i];
+      if (dw >= 0.0 && !((blocked >> qb) & 1u)) {
+        const double kap = (1.0 - 2.0 * dw) / (1.0 + 2.0 * dw);
+        val = val + kap * (fb - own);
+      }
+    } else if (p.has_uw) {
+      val = val + 6.0 * (q <= 6 ? 1.0 / 18.0 : 1.0 / 36.0) * (ax * p.wall_u[0] + ay * p.wall_u[1] + az * p.wall_u[2]);
+    }
+    f = val;
+  }
+  if (gasm) {
+    double rt = __shfl_sync(FULL, own, 0), j[3] = {0.0, 0.0, 0.0};
+    const double sum = fx_add(own, ownb), dif = (q & 1) ? fx_sub(own, ownb) : 0.0;
+#pragma unroll
+    for (int l = 1; l < 19; l += 2) {
+      const double e = __shfl_sync(FULL, dif, l);
+      rt = fx_add(rt, __shfl_sync(FULL, sum, l));
+      if (cx(l)) j[0] = fx_add(j[0], cx(l) * e);
+      if (cy(l)) j[1] = fx_add(j[1], cy(l) * e);
+      if (cz(l)) j[2] = fx_add(j[2], cz(l) * e);
+    }
+    Surface64 S;
+    surface64(p, v, li, rt, j, S);
+    // both lanes of a pair run its closure, as the thread does from the odd link
+    const bool odd = (q & 1) != 0;
+    const int sg = odd ? 1 : -1, qo = odd ? q : qb, qe = odd ? qb : q;
+    double fo = odd ? f : fb, fe = odd ? fb : f;
+    const bool ga = q && ((gasm >> qo) & 1u), gb = q && ((gasm >> qe) & 1u);
+    if (ga || gb) {
+      gas_pair64(p, S, q <= 6 ? 1.0 / 18.0 : 1.0 / 36.0, sg * ax, sg * ay, sg * az, odd ? own : ownb, odd ? ownb : own,
+                 ga, gb, (blocked >> qo) & 1u, (blocked >> qe) & 1u, fo, fe);
+      if ((gasm >> q) & 1u) f = odd ? fo : fe;
+    }
+  }
+  double rho;
+  long long rf;
+  if (!collide_warp(p, q, f, rf)) {  // out of the fixed-point range: as a thread, on every lane
+    double g[19], ux, uy, uz;
+#pragma unroll
+    for (int l = 0; l < 19; ++l) g[l] = __shfl_sync(FULL, f, l);
+    collide<double>(p, g, rho, ux, uy, uz);
+    if (lane == 0 && rho_bad<false>(rho)) atomicOr(v.err, ERRB_UNSTABLE);
+#pragma unroll
+    for (int l = 0; l < 19; ++l) f = l == q ? g[l] : f;
+  } else {
+    rho = double_of_fix(rf);
+  }
+  if (lane < 19) v.fout[(size_t)q * N + (size_t)i] = f;
+  return lane == 0 ? finish64(p, v, i, dm, rho, wallm, gasm, fill, empty) : 0.0;
 }
 
 // ---------------------------------------------------------------------------
@@ -511,7 +628,27 @@ __global__ void __launch_bounds__(128, (EXT ? 2 : (P == P64 ? 3 : 5))) k_iface(P
   const int stride = gridDim.x * blockDim.x;
   const int rounds = (count + stride - 1) / stride;
   double msum = 0.0;
+  if constexpr (LEAN) {
+    // A short list by a warp per cell: the thread's version is a chain of 24 us
+    // (16 cells of a 4x4x32 film, alone), this one of 11.5 us.  Above 8 cells an SM
+    // the warps' FP64 operations, as many for one cell as for 32, take longer.
+    if (count <= 152 * 8) {
+      const int lane = threadIdx.x & 31;
+      for (int e = (threadIdx.x >> 5) * gridDim.x + blockIdx.x; e < count; e += (blockDim.x >> 5) * gridDim.x) {
+        const int pos = e < n_in ? e : v.cap - 1 - (e - n_in);
+        const long long i = FSL_CK(p, v.ilist[pos], p.N);
+        int x, y, z;
+        coords(p, i, x, y, z);
+        bool fill = false, empty = false;
+        const double mm = iface_warp64(p, v, pos, i, x, y, z, fill, empty);
+        if (lane == 0 && owned(p, x, y, z)) msum += mm;
+        warp_append(lane == 0 && fill, (int)i, v.flist, &v.cnt[1], v.cap, v.err);
+        warp_append(lane == 0 && empty, (int)i, v.elist, &v.cnt[2], v.cap, v.err);
+      }
+    }
+  }
   for (int r = 0; r < rounds; ++r) {
+    if (LEAN && count <= 152 * 8) break;
     const int li = r * stride + blockIdx.x * blockDim.x + threadIdx.x;
     const bool act = li < count;
     bool fill = false, empty = false;
