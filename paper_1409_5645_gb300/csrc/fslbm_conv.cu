@@ -27,6 +27,7 @@
 #include "fslbm_dev.cuh"
 #include "fslbm_fixed.cuh"
 #include "fslbm_kernels.h"
+#include "fslbm_pull.cuh"
 
 namespace fsl {
 
@@ -341,6 +342,14 @@ __device__ __forceinline__ double split_weight(const double (&n)[3], int ax, int
   return filled ? (d > 0.0 ? d : 0.0) : (d < 0.0 ? -d : 0.0);
 }
 
+template <int P>
+__device__ __noinline__ double sender_weight(const Par& p, const View<P>& v, long long i, int ax, int ay, int az,
+                                             bool filled) {
+  double n[3];
+  fill_normal<P>(p, v, i, n);
+  return split_weight(n, ax, ay, az, filled);
+}
+
 // fill or empty cell k (of nf fills, then the empties) by a warp: lane q (1..18)
 // tests neighbour q as a receiver; lane 0 computes the share (rho summed in q
 // order, as a thread would)
@@ -375,9 +384,7 @@ __device__ __forceinline__ void share_cell(const Par& p, const View<P>& v, int k
     // weighted split: the receivers' weights summed in q order on lane 0
     double V = 0.0;
     if (p.excess_split && rm) {
-      double n[3];
-      fill_normal<P>(p, v, i, n);  // (every lane: the same few loads)
-      const double w = recv ? split_weight(n, cx(q), cy(q), cz(q), isF) : 0.0;
+      const double w = recv ? sender_weight<P>(p, v, i, cx(q), cy(q), cz(q), isF) : 0.0;
       for (int s = 1; s < 19; ++s) V += __shfl_sync(FULL, w, s);
     }
     if (lane == 0) {
@@ -423,18 +430,40 @@ __global__ void __launch_bounds__(256) k_new_share(Par p, View<P> v) {
   do_new_share<P>(p, v);
 }
 
+// a receiver's shares where some of them are split along the normal (out of
+// line: an option, and with its normals inlined for every link it was most of
+// the kernel's code)
+template <int P>
+__device__ __noinline__ double weighted_shares(const Par& p, const View<P>& v, int x, int y, int z) {
+  double acc = 0.0;
+#pragma unroll 1
+  for (int q = 1; q < 19; ++q) {
+    const long long j = nbr(p, x, y, z, cx(q), cy(q), cz(q));
+    const uint8_t mk = j < 0 ? (uint8_t)0 : v.mark[j];
+    if (!(mk & (MK_FILL | MK_EMPTY))) continue;
+    if (mk & MK_WSPLIT) {  // the link from j to this receiver is -c_q
+      double n[3];
+      fill_normal<P>(p, v, j, n);
+      acc += v.share[j] * split_weight(n, -cx(q), -cy(q), -cz(q), (mk & MK_FILL) != 0);
+    } else {
+      acc += v.share[j];
+    }
+  }
+  return acc;
+}
+
 // one thread per receiver (the lists are long late in a run): gathers the
 // shares of its converting neighbours in q order (deterministic)
 template <int P>
 __device__ __forceinline__ void do_recv(const Par& p, const View<P>& v) {
   using R = typename Form<P>::R;
   const LaneItems it(min(load_count(&v.cnt[5]), v.cap), grid_warp());
-  const long long sy = p.nx, sz = (long long)p.nx * p.ny;
   for (int k = it.k; k < it.end; k += it.step) {
     const long long yj = FSL_CK(p, v.rlist[k], p.N);
     int x, y, z;
     coords(p, yj, x, y, z);
-    const bool in1 = x >= 1 && x < p.nx - 1 && y >= 1 && y < p.ny - 1 && z >= 1 && z < p.nz - 1;
+    int src[19];
+    pull_sources(p, x, y, z, src);
     // the receiver's own mass and density first: their loads overlap the
     // neighbours' marks and shares
     const double m0 = v.m[yj];
@@ -443,34 +472,22 @@ __device__ __forceinline__ void do_recv(const Par& p, const View<P>& v) {
     // in flight together (a load, a test and a dependent load per neighbour in
     // turn took 13 us of a 128x64x64 splash's 41 us conversions)
     unsigned conv = 0u, wsp = 0u;
-    int jq[19];
 #pragma unroll
     for (int q = 1; q < 19; ++q) {
-      const long long j = in1 ? yj + (cx(q) + sy * cy(q) + sz * cz(q)) : nbr(p, x, y, z, cx(q), cy(q), cz(q));
-      jq[q] = (int)j;
+      const int j = src[inv(q)];  // x + c_q
       const uint8_t mk = j < 0 ? (uint8_t)0 : v.mark[j];
       if (mk & (MK_FILL | MK_EMPTY)) conv |= 1u << q;
       if (mk & MK_WSPLIT) wsp |= 1u << q;
     }
     double acc = 0.0, sh[19];
 #pragma unroll
-    for (int q = 1; q < 19; ++q) sh[q] = (conv & (1u << q)) ? v.share[jq[q]] : 0.0;
+    for (int q = 1; q < 19; ++q) sh[q] = (conv & (1u << q)) ? v.share[src[inv(q)]] : 0.0;
     if (!(conv & wsp)) {
 #pragma unroll
       for (int q = 1; q < 19; ++q)
         if (conv & (1u << q)) acc += sh[q];
     } else {
-#pragma unroll
-      for (int q = 1; q < 19; ++q) {
-        if (!(conv & (1u << q))) continue;
-        if (wsp & (1u << q)) {  // the link from j to this receiver is -c_q
-          double n[3];
-          fill_normal<P>(p, v, jq[q], n);
-          acc += sh[q] * split_weight(n, -cx(q), -cy(q), -cz(q), (v.mark[jq[q]] & MK_FILL) != 0);
-        } else {
-          acc += sh[q];
-        }
-      }
+      acc = weighted_shares<P>(p, v, x, y, z);
     }
     const double mm = m0 + acc;
     v.m[yj] = mm;
@@ -613,7 +630,7 @@ __device__ __forceinline__ void reduce_mass(const MassReduce& mr, int chunk, int
 // wait there.  A step without a fill or an empty cell has the mass only.
 // Alone, with warm caches: a film's step 17.2 -> 6.8 us without the barriers;
 // with conversions, a stage's items one to a warp over all SMs and a
-// receiver's loads together, a 128x64x64 splash's 46.8 -> 38.8 us, a 256x128x128 FP64
+// receiver's loads together, a 128x64x64 splash's 46.8 -> 35.9 us, a 256x128x128 FP64
 // splash's 96 -> 60 us
 template <int P>
 __global__ void __launch_bounds__(256) k_convert(Par p, View<P> v, MassReduce mr) {
