@@ -319,6 +319,10 @@ __device__ __forceinline__ double link_dot(int ax, int ay, int az, const double 
   return fx_fma((double)ax, a[0], fx_fma((double)ay, a[1], fx_mul((double)az, a[2])));
 }
 
+__device__ __forceinline__ float link_dot32(int ax, int ay, int az, float a0, float a1, float a2) {
+  return fx_fma((float)ax, a0, fx_fma((float)ay, a1, fx_mul((float)az, a2)));
+}
+
 // what the links of a cell share
 struct Surface64 {
   double n[3], d;        // the plane of k_geom
@@ -543,6 +547,163 @@ __device__ __forceinline__ double iface_warp64(const Par& p, const View<P64>& v,
   return lane == 0 ? finish64(p, v, i, dm, rho, wallm, gasm, fill, empty) : 0.0;
 }
 
+// The default interface cell of the FP32 and FP16 forms by a warp, link q on
+// lane q (the lanes from 19 on repeat the rest population and write nothing):
+// the operations and roundings of iface_cell<P, ., false>, sums in its order,
+// written out so that no compiler choice of fused multiply-adds separates the
+// two.  fill, empty and the returned mass are lane 0's.
+template <int P>
+__device__ __forceinline__ double iface_warp32(const Par& p, const View<P>& v, int li, long long i, int x, int y, int z,
+                                               bool& fill, bool& empty) {
+  static_assert(sizeof(typename Form<P>::R) == 4 && Form<P>::SH, "the reduced forms");
+  const unsigned FULL = 0xffffffffu;
+  const size_t N = (size_t)p.N;
+  const int lane = threadIdx.x & 31, q = lane < 19 ? lane : 0, qb = q == 0 ? 0 : ((q & 1) ? q + 1 : q - 1);
+  const int ax = cx(q), ay = cy(q), az = cz(q);
+  const long long s = nbr(p, x, y, z, -ax, -ay, -az);
+  const uint8_t ks = kind_at(v.flags, s);
+  const float own = ldq<P>(v.fin, (size_t)q * N + (size_t)i, q);
+  float f = ldq<P>(v.fin, (size_t)q * N + (size_t)(s < 0 ? 0 : s), q);
+  const float phic = v.phin[i], phs = s < 0 ? 0.f : v.phin[s];
+  if (!is_fluid(ks)) f = 0.f;
+  const bool link = lane >= 1 && lane < 19;
+  const unsigned wallm = __ballot_sync(FULL, link && ks == WALL);
+  const unsigned gasm = __ballot_sync(FULL, link && ks != WALL && !is_fluid(ks));
+  const unsigned blocked = wallm | gasm;
+  const float ownb = __shfl_sync(FULL, own, qb);
+  double dm = 0.0;
+  if (!p.freeze) {
+    const float sw = ks == LIQ ? 1.f : fx_mul(0.5f, fx_add(phic, phs)), flux = fx_mul(sw, fx_sub(f, ownb));
+#pragma unroll
+    for (int l = 1; l < 19; ++l) {
+      const float a = __shfl_sync(FULL, flux, l);
+      if (!((blocked >> l) & 1u)) dm += (double)a;
+    }
+  }
+  const float fb = __shfl_sync(FULL, f, qb);  // the opposite link's pulled value
+  if ((wallm >> q) & 1u) {                    // (wall_links)
+    float val = ownb;
+    if (p.has_wd) {
+      const float dw = (float)v.wd[(size_t)qb * N + (size_t)i];
+      if (dw >= 0.f && !((blocked >> qb) & 1u)) {
+        const float kap = __fdiv_rn(fx_fma(-2.f, dw, 1.f), fx_fma(2.f, dw, 1.f));
+        val = fx_fma(kap, fx_sub(fb, own), val);
+      }
+    } else if (p.has_uw) {
+      const float w6 = 6.f * (q <= 6 ? wq<float>(1) : wq<float>(7));
+      val = fx_fma(w6, link_dot32(ax, ay, az, (float)p.wall_u[0], (float)p.wall_u[1], (float)p.wall_u[2]), val);
+    }
+    f = val;
+  }
+  if (gasm) {
+    // the moments of the cell's own populations
+    float rt = 0.f, ux = 0.f, uy = 0.f, uz = 0.f;
+#pragma unroll
+    for (int l = 0; l < 19; ++l) {
+      const float a = __shfl_sync(FULL, own, l);
+      rt = fx_add(rt, a);
+      if (cx(l)) ux = cx(l) > 0 ? fx_add(ux, a) : fx_sub(ux, a);
+      if (cy(l)) uy = cy(l) > 0 ? fx_add(uy, a) : fx_sub(uy, a);
+      if (cz(l)) uz = cz(l) > 0 ? fx_add(uz, a) : fx_sub(uz, a);
+    }
+    const float ir0 = p.compressible ? 1.f / rho_full_r<true>(rt) : 1.f;
+    ux = fx_fma(ux, ir0, -fx_mul(0.5f, (float)p.g[0]));
+    uy = fx_fma(uy, ir0, -fx_mul(0.5f, (float)p.g[1]));
+    uz = fx_fma(uz, ir0, -fx_mul(0.5f, (float)p.g[2]));
+    float n0 = 0.f, n1 = 0.f, n2 = 0.f, d = 0.f, kap = 0.f;
+    if (p.rule != 0 || p.sigma != 0.0) {
+      const size_t cap = (size_t)v.cap;
+      n0 = v.geo[li];
+      n1 = v.geo[cap + li];
+      n2 = v.geo[2 * cap + li];
+      d = v.geo[3 * cap + li];
+      kap = v.geo[4 * cap + li];
+    }
+    float rb = (float)p.rho_G;
+    if (p.sigma != 0.0) rb = fx_fma((float)(3.0 * p.sigma), kap, rb);
+    const float r0b = p.compressible ? rb : 1.f, r0t = p.compressible ? rho_full_r<true>(rt) : 1.f;
+    rb = fx_sub(rb, 1.f);
+    if ((gasm >> q) & 1u) {
+      // boundary link p = qb (x + c_p is gas), rebuilt f_q
+      const float usq = fx_fma(uz, uz, fx_fma(ux, ux, fx_mul(uy, uy))), w = q <= 6 ? wq<float>(1) : wq<float>(7);
+      const float cu = link_dot32(-ax, -ay, -az, ux, uy, uz);
+      float eb = fx_mul(w, rb), et = fx_mul(w, rt);
+      if (!p.linear_eq) {
+        const float t = fx_fma(fx_mul(3.f, cu), cu, -usq);
+        eb = fx_fma(fx_mul(fx_mul(w, 1.5f), r0b), t, eb);
+        et = fx_fma(fx_mul(fx_mul(w, 1.5f), r0t), t, et);
+      }
+      if (p.rule == 0 || ((blocked >> qb) & 1u)) {
+        f = fx_fma(2.f, eb, -ownb);
+      } else {
+        float dl = 0.5f;
+        const float cn = link_dot32(-ax, -ay, -az, n0, n1, n2);
+        if (cn > 0.f) {
+          dl = qdiv(d, cn);
+          dl = dl < (float)p.delta_min ? (float)p.delta_min : (dl > 1.f ? 1.f : dl);
+        }
+        const float nplus = fx_mul(fx_fma(0.5f, fx_add(ownb, own), -et), (float)p.inv_1plp), lp = (float)p.lam_p;
+        const float C = fx_fma(lp, fx_add(0.5f, dl), -fx_mul(2.f, lp));
+        float r = fx_fma(fx_sub(0.5f, dl), ownb, fx_mul(0.5f, own));
+        r = fx_fma(fx_sub(dl, 1.f), fb, r);
+        r = fx_fma(C, nplus, r);
+        f = fx_add(r, eb);
+      }
+    }
+  }
+  // the collision (collide): moments in population order, then the link's pair
+  float r, jx = 0.f, jy = 0.f, jz = 0.f;
+  r = __shfl_sync(FULL, f, 0);
+#pragma unroll
+  for (int l = 1; l < 19; ++l) {
+    const float a = __shfl_sync(FULL, f, l);
+    r = fx_add(r, a);
+    if (cx(l)) jx = cx(l) > 0 ? fx_add(jx, a) : fx_sub(jx, a);
+    if (cy(l)) jy = cy(l) > 0 ? fx_add(jy, a) : fx_sub(jy, a);
+    if (cz(l)) jz = cz(l) > 0 ? fx_add(jz, a) : fx_sub(jz, a);
+  }
+  const float fo = __shfl_sync(FULL, f, qb);
+  const float r0 = p.compressible ? rho_full_r<true>(r) : 1.f, i0 = p.compressible ? 1.f / r0 : 1.f;
+  const float Ux = fx_mul(jx, i0), Uy = fx_mul(jy, i0), Uz = fx_mul(jz, i0);
+  const float gx = (float)p.g[0], gy = (float)p.g[1], gz = (float)p.g[2], ilm = (float)p.inv_lam_m;
+  const float ux = fx_fma(0.5f, gx, Ux), uy = fx_fma(0.5f, gy, Uy), uz = fx_fma(0.5f, gz, Uz);
+  const float vx = fx_fma(-gx, ilm, Ux), vy = fx_fma(-gy, ilm, Uy), vz = fx_fma(-gz, ilm, Uz);
+  const float usq = fx_fma(uz, uz, fx_fma(uy, uy, fx_mul(ux, ux)));
+  const float lp = (float)p.lam_p, lm = (float)p.lam_m, nl = p.linear_eq ? 0.f : 1.f;
+  const float w = q == 0 ? wq<float>(0) : (q <= 6 ? wq<float>(1) : wq<float>(7));
+  const float kw = fx_mul(fx_mul(1.5f * w, r0), nl);
+  float out;
+  if (q == 0) {
+    out = fx_fma(lp, fx_sub(f, fx_fma(kw, -usq, fx_mul(w, r))), f);
+  } else {
+    constexpr float m7f = 1.f / 12.f, m1f = (1.f - 8.f * m7f) * 0.5f;
+    const float mw = fx_mul(q <= 6 ? m1f : m7f, r0);
+    const bool odd = (q & 1) != 0;
+    const int sg = odd ? 1 : -1;  // (the pair's terms from its odd link)
+    const float fq = odd ? f : fo, fqb = odd ? fo : f;
+    const float cu = link_dot32(sg * ax, sg * ay, sg * az, ux, uy, uz);
+    const float cv = link_dot32(sg * ax, sg * ay, sg * az, vx, vy, vz);
+    const float ep = fx_fma(kw, fx_fma(fx_mul(3.f, cu), cu, -usq), fx_mul(w, r)), em = fx_mul(mw, cv);
+    const float np = fx_fma(0.5f, fx_add(fq, fqb), -ep), nm = fx_fma(0.5f, fx_sub(fq, fqb), -em);
+    out = fx_fma(odd ? lm : -lm, nm, fx_fma(lp, np, f));
+  }
+  if (lane < 19) stq<P>(v.fout, (size_t)q * N + (size_t)i, q, out);
+  if (lane != 0) return 0.0;
+  if (rho_bad<true>(r)) atomicOr(v.err, ERRB_UNSTABLE);
+  double mm = v.m[i];
+  if (!p.freeze) {
+    const double rhof = rho_full<true>(r);
+    mm = mm + dm;
+    v.m[i] = mm;
+    v.phout[i] = (float)(mm / rhof);
+    fill = mm > (1.0 + p.eps) * rhof || ((p.cleanup & 1) && gasm == 0u);
+    empty = !fill && (mm < -p.eps * rhof || ((p.cleanup & 2) && blocked == 0x7fffeu));
+    if (fill) v.mark[i] = MK_FILL;
+    else if (empty) v.mark[i] = MK_EMPTY;
+  }
+  return mm;
+}
+
 // ---------------------------------------------------------------------------
 // k_geom: plane (normal, offset) and curvature of every listed interface cell
 // from phi(t) (Sec. 2.2, Sec. 5) into v.geo; kept apart from k_iface so that
@@ -620,6 +781,15 @@ __global__ void __launch_bounds__(128) k_geom(Par p, View<P> v) {
 // and the normal links (separate, so that the default instance carries none
 // of their code).  LEAN: the FP64 form's instance with few FP64 operations
 // (where the fixed-point collision applies)
+//
+// A list of up to IFACE_WARP_MAX cells goes by a warp per cell, a longer one by
+// a thread per cell: the thread is a chain of 20 to 24 us however few cells
+// there are, the warp one of 11.5 us (16 FP64 cells of a 4x4x32 film, alone,
+// warm caches).  The line lies at 8 cells an SM: a warp's FP64 operations (in
+// the reduced forms those of the cell's mass) hold the FP64 pipe as long for
+// one cell as for 32, and 12.7 k FP32 cells of a 128x64x64 splash took 74 us by
+// warps against 20 us by threads.
+constexpr int IFACE_WARP_MAX = 152 * 8;
 template <int P, bool EXT, bool LEAN = false>
 __global__ void __launch_bounds__(128, (EXT ? 2 : (P == P64 ? 3 : 5))) k_iface(Par p, View<P> v, int part_base) {
   pdl_begin();
@@ -628,11 +798,11 @@ __global__ void __launch_bounds__(128, (EXT ? 2 : (P == P64 ? 3 : 5))) k_iface(P
   const int stride = gridDim.x * blockDim.x;
   const int rounds = (count + stride - 1) / stride;
   double msum = 0.0;
-  if constexpr (LEAN) {
-    // A short list by a warp per cell: the thread's version is a chain of 24 us
-    // (16 cells of a 4x4x32 film, alone), this one of 11.5 us.  Above 8 cells an SM
-    // the warps' FP64 operations, as many for one cell as for 32, take longer.
-    if (count <= 152 * 8) {
+  // a short list by a warp per cell (the default instances)
+  constexpr bool WARP = LEAN || (P != P64 && !EXT);
+  const bool warp = WARP && count <= IFACE_WARP_MAX;
+  if constexpr (WARP) {
+    if (warp) {
       const int lane = threadIdx.x & 31;
       for (int e = (threadIdx.x >> 5) * gridDim.x + blockIdx.x; e < count; e += (blockDim.x >> 5) * gridDim.x) {
         const int pos = e < n_in ? e : v.cap - 1 - (e - n_in);
@@ -640,7 +810,9 @@ __global__ void __launch_bounds__(128, (EXT ? 2 : (P == P64 ? 3 : 5))) k_iface(P
         int x, y, z;
         coords(p, i, x, y, z);
         bool fill = false, empty = false;
-        const double mm = iface_warp64(p, v, pos, i, x, y, z, fill, empty);
+        double mm;
+        if constexpr (P == P64) mm = iface_warp64(p, v, pos, i, x, y, z, fill, empty);
+        else mm = iface_warp32<P>(p, v, pos, i, x, y, z, fill, empty);
         if (lane == 0 && owned(p, x, y, z)) msum += mm;
         warp_append(lane == 0 && fill, (int)i, v.flist, &v.cnt[1], v.cap, v.err);
         warp_append(lane == 0 && empty, (int)i, v.elist, &v.cnt[2], v.cap, v.err);
@@ -648,7 +820,7 @@ __global__ void __launch_bounds__(128, (EXT ? 2 : (P == P64 ? 3 : 5))) k_iface(P
     }
   }
   for (int r = 0; r < rounds; ++r) {
-    if (LEAN && count <= 152 * 8) break;
+    if (warp) break;
     const int li = r * stride + blockIdx.x * blockDim.x + threadIdx.x;
     const bool act = li < count;
     bool fill = false, empty = false;

@@ -120,16 +120,18 @@ def test_fields_into_buffers_of_either_alignment(dims):
             assert (got[:off] == 7).all() and (got[off + n:] == 7).all(), (k, off)
 
 
-@pytest.mark.parametrize("rule,kw", [(1, {}), (0, {}), (1, dict(tau=1.7, magic=0.25)), (1, dict(linear_eq=1))])
-def test_interface_cells_by_warp_and_by_thread(rule, kw):
+@pytest.mark.parametrize("precision", ["f64", "f32", "f16"])
+@pytest.mark.parametrize("rule,kw", [(1, {}), (0, {}), (1, dict(tau=1.7, magic=0.25)), (1, dict(linear_eq=1)),
+                                     (1, dict(sigma=1e-3)), (0, dict(wall_u=(1e-3, 0.0, 0.0)))])
+def test_interface_cells_by_warp_and_by_thread(precision, rule, kw):
     """A lattice with more interface cells than the warp path takes, beside
     itself as two slabs that have fewer: the same bits after 20 steps with
     conversions."""
     c = cases.dam_break(nx=48, ny=40, nz=40, col_x=20, col_z=20, g=4e-4, rule=rule, phi_noise=0.3, **{"tau": 0.6, **kw})
     c["phi"] = np.where(c["flags"] == cases.INTERFACE, np.clip(c["phi"], 0.05, 0.999), c["phi"])
     assert int((c["flags"] == cases.INTERFACE).sum()) > 1216 > 28 * 40
-    whole = fslbm.Lattice.from_case(c, precision="f64")
-    parts = slabs.LocalSlabs(c, parts=2, axis=1, precision="f64")
+    whole = fslbm.Lattice.from_case(c, precision=precision)
+    parts = slabs.LocalSlabs(c, parts=2, axis=1, precision=precision)
     whole.step(20)
     for _ in range(20):
         parts.step(1)
