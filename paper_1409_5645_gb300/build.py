@@ -26,7 +26,8 @@ ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 SOURCES = ["fslbm_step.cu", "fslbm_step_p64.cu", "fslbm_step_p32.cu", "fslbm_step_p16.cu", "fslbm_conv.cu",
            "fslbm_state.cu", "fslbm_api.cu", "fslbm_adjoint.cu", "fslbm_adjoint_p64.cu", "fslbm_adjoint_p32.cu",
            "fslbm_adjoint_p16.cu", "fslbm_noalloc.cu", "fslbm_staged.cu", "fslbm_halo.cu", "fslbm_rate.cu",
-           "fslbm_pairs.cu", "fslbm_bulk64.cu"]
+           "fslbm_pairs.cu", "fslbm_bulk64.cu",
+           "fslbm_small.cu"]
 
 
 def nvcc() -> str:

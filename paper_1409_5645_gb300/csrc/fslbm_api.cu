@@ -220,6 +220,10 @@ extern "C" int fslbm_create_ex(const fslbm_params* prm, fslbm_t** out) {
     const int per_sm = h->prec == FSLBM_F64   ? convert_blocks_per_sm<P64>()
                        : h->prec == FSLBM_F32 ? convert_blocks_per_sm<P32>()
                                               : convert_blocks_per_sm<P16>();
+    if (coop && sms > 0 && small_ok(p, h->prec))
+      h->small_blocks = h->prec == FSLBM_F64   ? small_blocks<P64>(p, sms)
+                        : h->prec == FSLBM_F32 ? small_blocks<P32>(p, sms)
+                                               : small_blocks<P16>(p, sms);
     h->coop_blocks = (coop && per_sm > 0 && sms > 0) ? sms * (per_sm < 2 ? per_sm : 2) : 0;
   }
   h->red_blocks = 152;
@@ -229,7 +233,7 @@ extern "C" int fslbm_create_ex(const fslbm_params* prm, fslbm_t** out) {
             dalloc(h, (char**)&h->fA, 19 * Nn * store_bytes(h->prec) + 16) &&
             dalloc(h, (char**)&h->fB, 19 * Nn * store_bytes(h->prec) + 16) && dalloc(h, &h->m, Nn * 8) &&
             dalloc(h, (char**)&h->phiA, Nn * real_bytes(h->prec)) &&
-            dalloc(h, (char**)&h->phiB, Nn * real_bytes(h->prec)) && dalloc(h, &h->cnt, 16 * sizeof(int)) &&
+            dalloc(h, (char**)&h->phiB, Nn * real_bytes(h->prec)) && dalloc(h, &h->cnt, 48 * sizeof(int)) &&
             dalloc(h, &h->share, Nn * 8) && dalloc(h, (char**)&h->geo, 5 * Nn * real_bytes(h->prec)) &&
             dalloc(h, &h->partials, (size_t)h->nparts * 8) &&
             dalloc(h, &h->red, (size_t)(h->red_blocks + 2) * 8) && dalloc(h, &h->lost, 8) &&
@@ -252,7 +256,7 @@ extern "C" int fslbm_create_ex(const fslbm_params* prm, fslbm_t** out) {
   cudaMemsetAsync(h->m, 0, Nn * 8, h->st);
   cudaMemsetAsync(h->phiA, 0, Nn * real_bytes(h->prec), h->st);
   cudaMemsetAsync(h->phiB, 0, Nn * real_bytes(h->prec), h->st);
-  cudaMemsetAsync(h->cnt, 0, 16 * sizeof(int), h->st);
+  cudaMemsetAsync(h->cnt, 0, 48 * sizeof(int), h->st);
   cudaMemsetAsync(h->lost, 0, 8, h->st);
   cudaMemsetAsync(h->err, 0, 8, h->st);
   cudaMemsetAsync(h->step_mass, 0, 8, h->st);
@@ -415,7 +419,7 @@ static int begin_state(fslbm* h, const uint8_t* flags, const double* wall_delta,
   CK(cudaMemsetAsync(h->err, 0, 8, h->st), "memset");
   CK(cudaMemsetAsync(h->mark, 0, ((N + 3) & ~(size_t)3), h->st), "memset");
   CK(cudaMemsetAsync(h->lost, 0, 8, h->st), "memset");
-  CK(cudaMemsetAsync(h->cnt, 0, 16 * sizeof(int), h->st), "memset");
+  CK(cudaMemsetAsync(h->cnt, 0, 48 * sizeof(int), h->st), "memset");
   if (launch_prepare_flags(h->par, h->flags, h->err, h->st)) return fail(h, FSLBM_ERR_CUDA, "prepare flags launch");
   if ((wall_delta != nullptr) != (h->par.has_wd != 0)) fslbm_drop_graphs(h);
   if (wall_delta) {
@@ -664,6 +668,24 @@ static bool graph_steps(fslbm* h, int steps) {
   return true;
 }
 
+// `steps` steps of a small lattice in one launch (fslbm_small.cu); false: not done
+template <int P>
+static bool small_t(fslbm* h, int steps) {
+  return launch_small<P>(h->par, make_view<P>(h), h->st, h->small_blocks, steps, (unsigned*)&h->cnt[12]) == 0;
+}
+static bool small_steps(fslbm* h, int steps) {
+  const bool ok = h->prec == FSLBM_F64   ? small_t<P64>(h, steps)
+                  : h->prec == FSLBM_F32 ? small_t<P32>(h, steps)
+                                         : small_t<P16>(h, steps);
+  if (!ok) {
+    cudaGetLastError();
+    h->small_blocks = 0;
+    return false;
+  }
+  h->cur ^= steps & 1;
+  return true;
+}
+
 extern "C" int fslbm_step(fslbm_t* h, int n) {
   if (!h || n < 0) return FSLBM_ERR_ARG;
   bool graphs = !h->graph_off && !h->timing;
@@ -675,7 +697,16 @@ extern "C" int fslbm_step(fslbm_t* h, int n) {
     }
     graphs = graphs && s == cudaStreamCaptureStatusNone;
   }
-  for (int s = 0; s < n;) {
+  int s0 = 0;
+  // a small lattice: all but the last step in launches of up to SMALL_STEPS
+  constexpr int SMALL_STEPS = 256, SMALL_LEAST = 4;
+  while (graphs && h->small_blocks > 0 && !(h->fp64_chain && h->prec == FSLBM_F64) && n - s0 > SMALL_LEAST) {
+    const int k = n - s0 - 1 < SMALL_STEPS ? n - s0 - 1 : SMALL_STEPS;
+    if (!small_steps(h, k)) break;
+    s0 += k;
+    h->t += k;
+  }
+  for (int s = s0; s < n;) {
     const int k = n - s >= GRAPH_STEPS ? GRAPH_STEPS : 1;
     graphs = graphs && !h->graph_off;
     if (graphs && graph_steps(h, k)) {

@@ -267,7 +267,8 @@ struct View {
   int* rlist;   // excess receivers
   int* cnt;     // [0] ilist front [6] ilist back [1] flist [2] elist [3] ng [4] nl [5] rl [7] emptied;
                 // [8] all conversions since set; [9] fluid segments; [10] grid barrier of k_convert;
-                // [11] blocks of it that have summed their chunk of the mass
+                // [11] blocks of it that have summed their chunk of the mass; [12] grid barrier of
+                // k_steps, [16..47] its two sets of step counters
   int cap;
   double* share;
   R* geo;            // interface geometry per list entry: [5][cap] n0, n1, n2, d, kappa (n = 0: none)

@@ -36,6 +36,7 @@ struct fslbm {
   double* partials;
   long long nparts;
   int bulk_blocks, iface_blocks, list_blocks, red_blocks;
+  int small_blocks;  // blocks of the many-steps kernel (0: not used)
   int coop_blocks;  // blocks of the fused cooperative conversion kernel (0: four launches)
   double* red;
   double* lost;

@@ -101,6 +101,16 @@ int convert_blocks_per_sm();
 int launch_reduce(const double* in, long long n, double* tmp, int tmp_blocks, const double* add, double* out,
                   cudaStream_t st);
 
+// many steps of a small lattice in one cooperative launch (fslbm_small.cu):
+// whether it takes the lattice, its grid (0: not usable), the launch (ctr: its
+// barrier's counter)
+constexpr long long SMALL_CELLS = 1LL << 16;
+bool small_ok(const Par& p, int prec);
+template <int P>
+int small_blocks(const Par& p, int sms);
+template <int P>
+int launch_small(const Par& p, const View<P>& v, cudaStream_t st, int blocks, int steps, unsigned* ctr);
+
 // state set-up and read-back (fslbm_state.cu)
 template <int P>
 int launch_init_pre(const Par& p, const View<P>& v, const double* f, const double* phi, const double* rho_in,
