@@ -1215,7 +1215,16 @@ int adj_backward(fslbm* h) {
                       A->ck_flags + s * N))
       return 1;
     int n = A->nsteps - s * A->K < A->K ? A->nsteps - s * A->K : A->K;
-    for (int k = 0; k <= n; ++k) {  // the states before each step and after the last
+    // the states before each step and after the last; a small lattice's in
+    // one launch but for the last step, whose kernels leave the counters
+    int k0 = 0;
+    if (n > 1) {
+      if (save_state(h, A->seg_f, A->seg_m, A->seg_phi, A->seg_flags)) return 1;
+      h->fp64_chain = 1;
+      if (fslbm_logged_steps(h, n - 1, StateLog{A->seg_f, A->seg_m, A->seg_phi, A->seg_flags})) k0 = n - 1;
+      h->fp64_chain = 0;
+    }
+    for (int k = k0; k <= n; ++k) {
       if (save_state(h, (char*)A->seg_f + k * A->fbytes, A->seg_m + k * N, (char*)A->seg_phi + k * A->rbytes,
                      A->seg_flags + k * N))
         return 1;

@@ -2,9 +2,10 @@
 //
 // A handle owns every device buffer of one lattice.  fslbm_step enqueues, per
 // time step and with no host synchronisation:
-//   memset(counters) -> k_segments -> k_bulk -> k_iface -> mass reduction
-//   (2 kernels) -> 7 conversion kernels (dynamic interface only)
-// and swaps the A/B population and fill-level buffers.
+//   k_reset -> k_segments -> [bulk kernel beside k_geom -> k_iface] ->
+//   k_convert (with the mass reduction)
+// by graphs of eight steps or one, or, on a small lattice, all but the last
+// step in k_steps, and swaps the A/B population and fill-level buffers.
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stdio.h>
@@ -670,13 +671,15 @@ static bool graph_steps(fslbm* h, int steps) {
 
 // `steps` steps of a small lattice in one launch (fslbm_small.cu); false: not done
 template <int P>
-static bool small_t(fslbm* h, int steps) {
-  return launch_small<P>(h->par, make_view<P>(h), h->st, h->small_blocks, steps, (unsigned*)&h->cnt[12]) == 0;
+static bool small_t(fslbm* h, int steps, const StateLog& log) {
+  Par par = h->par;
+  if (h->fp64_chain) par.fix_ok = 0;
+  return launch_small<P>(par, make_view<P>(h), h->st, h->small_blocks, steps, (unsigned*)&h->cnt[12], log) == 0;
 }
-static bool small_steps(fslbm* h, int steps) {
-  const bool ok = h->prec == FSLBM_F64   ? small_t<P64>(h, steps)
-                  : h->prec == FSLBM_F32 ? small_t<P32>(h, steps)
-                                         : small_t<P16>(h, steps);
+static bool small_steps(fslbm* h, int steps, const StateLog& log) {
+  const bool ok = h->prec == FSLBM_F64   ? small_t<P64>(h, steps, log)
+                  : h->prec == FSLBM_F32 ? small_t<P32>(h, steps, log)
+                                         : small_t<P16>(h, steps, log);
   if (!ok) {
     cudaGetLastError();
     h->small_blocks = 0;
@@ -686,23 +689,34 @@ static bool small_steps(fslbm* h, int steps) {
   return true;
 }
 
+// the handle's stream takes whole graphs and many-steps launches now
+static bool whole_steps(fslbm* h) {
+  if (h->graph_off || h->timing) return false;
+  cudaStreamCaptureStatus s = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(h->st, &s) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return s == cudaStreamCaptureStatusNone;
+}
+
+// n steps of a small lattice in one launch, the state after step k (1 .. n) at
+// slot k of the log; false: not done
+bool fslbm_logged_steps(fslbm* h, int n, const StateLog& log) {
+  if (n < 1 || h->small_blocks <= 0 || !whole_steps(h) || !small_steps(h, n, log)) return false;
+  h->t += n;
+  return true;
+}
+
 extern "C" int fslbm_step(fslbm_t* h, int n) {
   if (!h || n < 0) return FSLBM_ERR_ARG;
-  bool graphs = !h->graph_off && !h->timing;
-  if (graphs) {
-    cudaStreamCaptureStatus s = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(h->st, &s) != cudaSuccess) {
-      cudaGetLastError();
-      graphs = false;
-    }
-    graphs = graphs && s == cudaStreamCaptureStatusNone;
-  }
+  bool graphs = whole_steps(h);
   int s0 = 0;
   // a small lattice: all but the last step in launches of up to SMALL_STEPS
   constexpr int SMALL_STEPS = 256, SMALL_LEAST = 4;
-  while (graphs && h->small_blocks > 0 && !(h->fp64_chain && h->prec == FSLBM_F64) && n - s0 > SMALL_LEAST) {
+  while (graphs && h->small_blocks > 0 && n - s0 > SMALL_LEAST) {
     const int k = n - s0 - 1 < SMALL_STEPS ? n - s0 - 1 : SMALL_STEPS;
-    if (!small_steps(h, k)) break;
+    if (!small_steps(h, k, StateLog{})) break;
     s0 += k;
     h->t += k;
   }

@@ -66,6 +66,8 @@ struct fslbm {
   int graph_off;         // a capture or a graph launch failed: steps are launched one kernel at a time
 };
 
+// many steps of a small lattice with every state logged (fslbm_api.cu); false: not done
+bool fslbm_logged_steps(fslbm* h, int n, const fsl::StateLog& log);
 // the captured steps hold the parameters by value: to be called when they change
 void fslbm_drop_graphs(fslbm* h);
 

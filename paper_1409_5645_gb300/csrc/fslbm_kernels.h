@@ -108,8 +108,17 @@ constexpr long long SMALL_CELLS = 1LL << 16;
 bool small_ok(const Par& p, int prec);
 template <int P>
 int small_blocks(const Par& p, int sms);
+// where the state after each step goes (the segment buffers of a reverse
+// sweep: state k at f + k 19 N and so on), or f = NULL
+struct StateLog {
+  void* f;
+  double* m;
+  void* phi;
+  uint8_t* flags;
+};
 template <int P>
-int launch_small(const Par& p, const View<P>& v, cudaStream_t st, int blocks, int steps, unsigned* ctr);
+int launch_small(const Par& p, const View<P>& v, cudaStream_t st, int blocks, int steps, unsigned* ctr,
+                 const StateLog& log);
 
 // state set-up and read-back (fslbm_state.cu)
 template <int P>

@@ -65,8 +65,12 @@ __device__ __noinline__ void liquid_cell(const Par& p, const View<P>& v, long lo
   for (int q = 0; q < 19; ++q) stq<P>(v.fout, (size_t)q * N + (size_t)i, q, f[q]);
 }
 
-template <int P, bool SIG>
-__global__ void __launch_bounds__(256, 1) k_steps(Par p, View<P> v, int steps, unsigned* ctr) {
+// CHAIN: the FP64 form without the fixed-point collision (the steps of a
+// differentiation, whose operations stay those they have always been): the
+// interface cell is the thread's general one.
+// log: the state after every step is also copied there.
+template <int P, bool SIG, bool CHAIN>
+__global__ void __launch_bounds__(256, 1) k_steps(Par p, View<P> v, int steps, unsigned* ctr, StateLog log) {
   using R = typename Form<P>::R;
   using S = typename Form<P>::S;
   const int lane = threadIdx.x & 31, nw = grid_warps(), wid = grid_warp();
@@ -120,8 +124,19 @@ __global__ void __launch_bounds__(256, 1) k_steps(Par p, View<P> v, int steps, u
         __syncwarp();
       }
       bool fill = false, empty = false;
-      if constexpr (P == P64) iface_warp64(p, v, e, i, x, y, z, fill, empty);
-      else iface_warp32<P>(p, v, e, i, x, y, z, fill, empty);
+      if constexpr (CHAIN) {
+        if (lane == 0) {
+          if (x >= 3 && x < p.nx - 3 && y >= 3 && y < p.ny - 3 && z >= 3 && z < p.nz - 3)
+            iface_cell<P, true, false>(p, v, e, i, x, y, z, fill, empty);
+          else
+            iface_cell<P, false, false>(p, v, e, i, x, y, z, fill, empty);
+        }
+        __syncwarp();
+      } else if constexpr (P == P64) {
+        iface_warp64(p, v, e, i, x, y, z, fill, empty);
+      } else {
+        iface_warp32<P>(p, v, e, i, x, y, z, fill, empty);
+      }
       warp_append(lane == 0 && fill, (int)i, v.flist, &v.cnt[1], v.cap, v.err);
       warp_append(lane == 0 && empty, (int)i, v.elist, &v.cnt[2], v.cap, v.err);
     }
@@ -151,6 +166,19 @@ __global__ void __launch_bounds__(256, 1) k_steps(Par p, View<P> v, int steps, u
     S* in = const_cast<S*>(v.fin);
     v.fin = v.fout;
     v.fout = in;
+    if (log.f) {
+      const long long n19 = 19 * p.N, at = (long long)(s + 1) * p.N;
+      const int t = wid * 32 + lane, nt = nw * 32;
+      S* lf = (S*)log.f + 19 * at;
+      R* lp = (R*)log.phi + at;
+      for (long long k = t; k < n19; k += nt) lf[k] = v.fin[k];
+      for (long long k = t; k < p.N; k += nt) {
+        log.m[at + k] = v.m[k];
+        lp[k] = v.phin[k];
+        log.flags[at + k] = v.flags[k];
+      }
+      if (!barrier()) return;  // the next step writes masses and kinds in place
+    }
   }
 }
 
@@ -164,6 +192,7 @@ __global__ void __launch_bounds__(256, 1) k_steps(Par p, View<P> v, int steps, u
 // IFACE_WARP_MAX) would set the step.
 bool small_ok(const Par& p, int prec) {
   if (p.stress || p.ub_extrap || p.recon_nc || p.elvira) return false;
+  // (an FP64 lattice whose equilibria or forces rule the fixed point out takes the kernels)
   if (prec == P64 && !p.fix_ok) return false;
   return p.N <= SMALL_CELLS;
 }
@@ -171,14 +200,20 @@ bool small_ok(const Par& p, int prec) {
 template <int P>
 int small_blocks(const Par& p, int sms) {
   int nb = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_steps<P, false>, 256, 0) != cudaSuccess || nb < 1) return 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_steps<P, true>, 256, 0) != cudaSuccess || nb < 1) return 0;
+  auto fits = [&](auto k) {
+    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k, 256, 0) == cudaSuccess && nb >= 1;
+  };
+  if (!fits(k_steps<P, false, false>) || !fits(k_steps<P, true, false>)) return 0;
+  if constexpr (P == P64) {
+    if (!fits(k_steps<P, false, true>)) return 0;
+  }
   const long long want = (p.N + 127) / 128;
   return (int)(want < 8 ? (sms < 8 ? sms : 8) : (want < sms ? want : sms));
 }
 
 template <int P>
-int launch_small(const Par& p, const View<P>& v, cudaStream_t st, int blocks, int steps, unsigned* ctr) {
+int launch_small(const Par& p, const View<P>& v, cudaStream_t st, int blocks, int steps, unsigned* ctr,
+                 const StateLog& log) {
   if (cudaMemsetAsync(ctr, 0, sizeof *ctr, st) != cudaSuccess) return 1;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(blocks);
@@ -189,13 +224,19 @@ int launch_small(const Par& p, const View<P>& v, cudaStream_t st, int blocks, in
   at[0].val.cooperative = 1;
   cfg.attrs = at;
   cfg.numAttrs = 1;
-  auto k = p.sigma != 0.0 ? k_steps<P, true> : k_steps<P, false>;
-  return (int)cudaLaunchKernelEx(&cfg, k, p, v, steps, ctr);
+  auto k = p.sigma != 0.0 ? k_steps<P, true, false> : k_steps<P, false, false>;
+  if constexpr (P == P64) {
+    if (!p.fix_ok) {
+      if (p.sigma != 0.0) return 1;
+      k = k_steps<P, false, true>;
+    }
+  }
+  return (int)cudaLaunchKernelEx(&cfg, k, p, v, steps, ctr, log);
 }
 
 #define FSL_INST(P)                                                                                       \
   template int small_blocks<P>(const Par&, int);                                                         \
-  template int launch_small<P>(const Par&, const View<P>&, cudaStream_t, int, int, unsigned*);
+  template int launch_small<P>(const Par&, const View<P>&, cudaStream_t, int, int, unsigned*, const StateLog&);
 FSL_INST(P64)
 FSL_INST(P32)
 FSL_INST(P16)

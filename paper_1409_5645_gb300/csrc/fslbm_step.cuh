@@ -2,11 +2,12 @@
 // segment scan k_segments, which lists the step's segments and interface
 // cells before them, is in fslbm_step.cu).
 //
-// k_bulk   every warp walks the segment list on its own, one lane per cell.
+// k_bulk   (FP32/FP16; the FP64 form's is in fslbm_bulk64.cu) every warp walks
+//          the segment list on its own, one lane per cell.
 //          Liquid cells pull their 19 populations (Eq. lbe1), apply half-way
 //          bounce-back / CLI at walls, collide (Eq. lbe2) and store.  The
 //          liquid density is reduced per warp for the mass balance.
-// k_iface  one thread per interface cell (grid-stride over the list): pulls,
+// k_iface  one thread (short lists: one warp) per interface cell: pulls,
 //          rebuilds the populations arriving from gas cells by the FSK rule
 //          (Eq. koerner) or the FSL rule (Eq. closure, Table 1, D = 0) with the
 //          link fraction from the height-function plane (Sec. 2.2, Sec. 5),
