@@ -235,7 +235,10 @@ int fslbm_set_state_post(fslbm_t *h, const uint8_t *flags, const double *f_post,
                          const double *phi, const double *wall_delta, int where);
 
 /* Advance n >= 0 time steps.  Asynchronous on the handle's stream: returns
- * launch errors only; method faults appear at the next synchronising call. */
+ * launch errors only; method faults appear at the next synchronising call.
+ * One call of n steps gives the bits of n calls of one step and costs less
+ * host time (steps go out as CUDA graphs, or many in one launch on a small
+ * lattice; the graphs belong to the handle). */
 int fslbm_step(fslbm_t *h, int n);
 
 /* Wait for the handle's stream; return the sticky device error, if any. */
@@ -296,7 +299,9 @@ enum fslbm_objective {
 /* Forward pass: run nsteps >= 1 steps from the current state with a full
  * checkpoint (flags, f~, m, phi) every K >= 1 steps, and return J.  Holds
  * ceil(nsteps/K) checkpoints on the device until the handle's state is set
- * again or the handle is destroyed. */
+ * again or the handle is destroyed; device buffers of up to 2 GiB in all stay
+ * with the handle after a new state, for the next differentiation with the
+ * same K and number of checkpoints. */
 int fslbm_adjoint_forward(fslbm_t *h, int nsteps, int K, int objective, double *J);
 
 /* Reverse pass (once per forward pass): recompute each K-step segment from
