@@ -727,8 +727,14 @@ template <int P>
 constexpr int geom_warp_max() { return P == P64 ? 2432 : 49152; }
 // SIG: the instance that also computes the curvature (surface tension); ELV:
 // the one with the ELVIRA normal where the height columns are open
+// The thread path waits for the gathers of its cell, so blocks in flight beside
+// the bulk kernel count for more than registers: 10 an SM for FP16 (48 registers,
+// from 64 and 128: a pass of a 128^3 wave 5.02 -> 4.79 ms, of a 512x256x256 splash
+// 17.36 -> 17.23) and 9 for plain FP32 (56: 19.38 -> 19.08).  FP64 keeps the
+// compiler's choice (5 blocks: a splash 7.26 -> 7.37 ms), FP32 with surface tension
+// or the elevation form has no measurement for a bound (0: none).
 template <int P, bool SIG, bool ELV>
-__global__ void __launch_bounds__(128) k_geom(Par p, View<P> v) {
+__global__ void __launch_bounds__(128, P == P16 ? 10 : P == P64 || SIG || ELV ? 0 : 9) k_geom(Par p, View<P> v) {
   pdl_begin();
   using R = typename Form<P>::R;
   const int n_in = min(*((volatile int*)&v.cnt[0]), v.cap), n_edge = min(*((volatile int*)&v.cnt[6]), v.cap - n_in);
