@@ -43,14 +43,18 @@ constexpr unsigned FULL = 0xffffffffu;
 template <int P>
 constexpr int pairs_blocks() { return P == P16 ? FSL_PAIRS_BLOCKS16 : FSL_PAIRS_BLOCKS32; }
 // blocks per SM in the launch when the interface kernels run beside it on
-// the side stream: fewer than resident, so that their blocks find room
-// (measured on the 512x256x256 dam break: FP32 at 3 of 5 and FP16 at 4 of 6
-// gave the shortest step)
+// the side stream: fewer than resident, so that their blocks find room; one
+// more of them ends at once where the step has more interface cells than
+// segments (few, below), for there the interface work sets the step.  Measured
+// on 512x256x256, FP32 / FP16, 3 and 4 blocks against 4 and 5: the dam break's
+// step with fewer interface cells than segments 0.417 / 0.355 -> 0.376 / 0.325
+// ms; a splash of 268 k interface cells, whole pass, 19.34 / 17.28 -> 19.76 /
+// 17.77 ms.  Near the line (300x130x120) the two differ by less than 1 %
 #ifndef FSL_PAIRS_GRID16
-#define FSL_PAIRS_GRID16 4
+#define FSL_PAIRS_GRID16 5
 #endif
 #ifndef FSL_PAIRS_GRID32
-#define FSL_PAIRS_GRID32 3
+#define FSL_PAIRS_GRID32 4
 #endif
 template <int P>
 constexpr int pairs_grid() { return P == P16 ? FSL_PAIRS_GRID16 : FSL_PAIRS_GRID32; }
@@ -231,7 +235,8 @@ __device__ __forceinline__ typename PairWord<P>::W pull_pair(const Par& p, const
 template <int P>
 __global__ void __launch_bounds__(128, pairs_blocks<P>()) k_bulk_pairs(Par p, View<P> v,
                                                                       const int* __restrict__ seglist,
-                                                                      const int* __restrict__ segcount, int nparts) {
+                                                                      const int* __restrict__ segcount, int nparts,
+                                                                      int few) {
   pdl_begin();
   using R = typename Form<P>::R;
   using PW = PairWord<P>;
@@ -239,8 +244,12 @@ __global__ void __launch_bounds__(128, pairs_blocks<P>()) k_bulk_pairs(Par p, Vi
   constexpr bool SH = Form<P>::SH;
   const int nseg = *((volatile const int*)segcount);
   const int lane = threadIdx.x & 31, hl = lane & 15;
+  // (few < grid: the blocks that stay where interface cells outnumber the segments)
+  const int nif = *((volatile const int*)&v.cnt[0]) + *((volatile const int*)&v.cnt[6]);
+  const int blocks = nif > nseg ? few : (int)gridDim.x;
+  if ((int)blockIdx.x >= blocks) return;
   const int gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int nw = (gridDim.x * blockDim.x) >> 5;
+  const int nw = (blocks * (int)blockDim.x) >> 5;
   const unsigned Nu = (unsigned)p.N, syu = (unsigned)p.nx, szu = (unsigned)(p.nx * p.ny);
   double msum = 0.0;
   // records and masks of the segment list (see k_segments); the next round's
@@ -331,7 +340,8 @@ int launch_bulk_pairs(const Par& p, const View<P>& v, cudaStream_t st, int bulk_
     // bulk_blocks is 8 resident blocks per SM of k_bulk; one resident wave
     // here, or fewer blocks beside the interface kernels (shared)
     const int grid = bulk_blocks / 8 * (shared ? pairs_grid<P>() : pairs_blocks<P>());
-    return launch_k(k_bulk_pairs<P>, grid, 128, 0, st, p, v, seglist, segcount, bulk_blocks * 4);
+    const int few = shared ? bulk_blocks / 8 * (pairs_grid<P>() - 1) : grid;
+    return launch_k(k_bulk_pairs<P>, grid, 128, 0, st, p, v, seglist, segcount, bulk_blocks * 4, few);
   }
 }
 

@@ -140,3 +140,20 @@ def test_interface_cells_by_warp_and_by_thread(precision, rule, kw):
     assert whole.counters()[4] > 0
     for k in a:
         assert np.array_equal(a[k].reshape(-1), np.asarray(b[k]).reshape(-1)), k
+
+
+@pytest.mark.parametrize("precision", ["f32", "f16"])
+@pytest.mark.parametrize("depth,more", [(80, False), (10, True)])
+def test_pair_kernel_grids_beside_the_interface_kernels(precision, depth, more):
+    """Fewer and more interface cells than segments of 32 cells (the pair
+    kernel keeps fewer blocks where there are more), beside every kernel in
+    order on the full grid."""
+    c = cases.dam_break(nx=512, ny=6, nz=96, col_x=500, col_z=depth, tau=0.6, g=2e-4, rule=1)
+    liquid = (c["flags"] == cases.LIQUID).reshape(-1, 32).any(1).sum()
+    assert ((c["flags"] == cases.INTERFACE).sum() > liquid) == more
+    a, b = (fslbm.Lattice.from_case(c, precision=precision, bulk_loads="pairs") for _ in range(2))
+    b.set_overlap(False)
+    for g in (a, b):
+        g.step(30)
+    assert _same(a, b) and a.counters()[4] > 0
+    assert a.step_mass() == pytest.approx(b.step_mass(), rel=1e-12)
