@@ -119,14 +119,13 @@ void fslbm_end_adjoint(fslbm* h) {
   h->adj->ready = h->adj->live = false;
 }
 
-static bool amalloc(AdjointState* A, void** p, size_t bytes) {
-  if (cudaMalloc(p, bytes ? bytes : 16) != cudaSuccess) {
-    *p = nullptr;
-    return false;
-  }
-  A->bytes += bytes;
-  return true;
+static bool amalloc(void** p, size_t bytes) {
+  if (cudaMalloc(p, bytes) == cudaSuccess) return true;
+  cudaGetLastError();  // (reported by the caller; the next launch must not find it)
+  *p = nullptr;
+  return false;
 }
+static void arelease(void* p) { cudaFree(p); }
 
 int save_state(fslbm* h, void* f, double* m, void* phi, uint8_t* flags) {
   AdjointState* A = h->adj;
@@ -175,10 +174,11 @@ extern "C" int fslbm_adjoint_forward(fslbm_t* h, int nsteps, int K, int objectiv
   const size_t sb = h->prec == FSLBM_F64 ? 8 : (h->prec == FSLBM_F32 ? 4 : 2);
   A->fbytes = 19 * N * sb;
   A->rbytes = N * (h->prec == FSLBM_F64 ? 8 : 4);
-  bool ok = kept || (amalloc(A, &A->ck_f, A->fbytes * A->nck) && amalloc(A, (void**)&A->ck_m, N * 8 * A->nck) &&
-            amalloc(A, &A->ck_phi, A->rbytes * A->nck) && amalloc(A, (void**)&A->ck_flags, N * A->nck) &&
-            amalloc(A, (void**)&A->red, ADJ_RED_DOUBLES * 8));
-  if (!ok) {
+  if (!kept && !adj_alloc_all(A,
+                              {{&A->ck_f, A->fbytes * nck}, {(void**)&A->ck_m, N * 8 * nck},
+                               {&A->ck_phi, A->rbytes * nck}, {(void**)&A->ck_flags, N * nck},
+                               {(void**)&A->red, ADJ_RED_DOUBLES * 8}},
+                              amalloc, arelease)) {
     fslbm_free_adjoint(h);
     return adj_fail(h, FSLBM_ERR_OOM, "adjoint checkpoint allocation");
   }
@@ -228,19 +228,8 @@ extern "C" int fslbm_adjoint_backward(fslbm_t* h, double* dJ_dnu, double dJ_dg[3
   AdjointState* A = h->adj;
   if (!A || !A->ready) return adj_fail(h, FSLBM_ERR_ARG, "fslbm_adjoint_forward has not run");
   const size_t N = (size_t)h->par.N;
-  if (!A->abar[0]) {
-    bool ok = amalloc(A, (void**)&A->abar[0], 19 * N * 8) && amalloc(A, (void**)&A->abar[1], 19 * N * 8) &&
-              amalloc(A, (void**)&A->P, 19 * N * 8) && amalloc(A, (void**)&A->mbar[0], N * 8) &&
-              amalloc(A, (void**)&A->mbar[1], N * 8) && amalloc(A, (void**)&A->phibar[0], N * 8) &&
-              amalloc(A, (void**)&A->phibar[1], N * 8) && amalloc(A, (void**)&A->theta, 64) &&
-              amalloc(A, (void**)&A->dphi0, N * 8) && amalloc(A, &A->seg_f, A->fbytes * (A->K + 1)) &&
-              amalloc(A, (void**)&A->seg_m, N * 8 * (A->K + 1)) &&
-              amalloc(A, &A->seg_phi, A->rbytes * (A->K + 1)) &&
-              amalloc(A, (void**)&A->seg_flags, N * (A->K + 1)) && amalloc(A, (void**)&A->Mh, N * 8) &&
-              amalloc(A, (void**)&A->flist, 2 * (2 * N + 2) * sizeof(int)) &&
-              amalloc(A, (void**)&A->rh, N * 8) && amalloc(A, (void**)&A->ngb, N * 4 * 8);
-    if (!ok) return adj_fail(h, FSLBM_ERR_OOM, "adjoint buffer allocation");
-  }
+  if (!adj_alloc_reverse(A, N, amalloc, arelease))
+    return adj_fail(h, FSLBM_ERR_OOM, "adjoint buffer allocation");
   int r;
   switch (h->prec) {
     case FSLBM_F64: r = adj_backward<P64>(h); break;

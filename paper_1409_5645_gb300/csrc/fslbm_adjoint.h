@@ -5,6 +5,7 @@
 #pragma once
 #include <cuda_runtime.h>
 #include <stdint.h>
+#include <initializer_list>
 
 #include "fslbm.h"
 #include "fslbm_dev.cuh"
@@ -41,8 +42,50 @@ struct AdjointState {
   double fwd_ms = 0.0, adj_ms = 0.0;
   size_t bytes = 0;
   bool ready = false;
+  bool reverse = false;  // every buffer of the reverse sweep is allocated (adj_alloc_reverse)
   bool live = false;  // belongs to the handle's current state (a new state ends it, its buffers may stay)
 };
+
+struct AdjBuffer {
+  void** p;
+  size_t bytes;
+};
+// All of the buffers (null before) or none: where one cannot be had, those
+// before it are given back and null again.  (alloc: pointer to fill, bytes ->
+// done, null where not; release: pointer)
+template <class Alloc, class Release>
+inline bool adj_alloc_all(AdjointState* A, std::initializer_list<AdjBuffer> bufs, Alloc alloc, Release release) {
+  for (const AdjBuffer* b = bufs.begin(); b != bufs.end(); ++b) {
+    if (alloc(b->p, b->bytes ? b->bytes : 16)) {
+      A->bytes += b->bytes;
+      continue;
+    }
+    while (b != bufs.begin()) {
+      --b;
+      release(*b->p);
+      *b->p = nullptr;
+      A->bytes -= b->bytes;
+    }
+    return false;
+  }
+  return true;
+}
+// the buffers of the reverse sweep, once per state
+template <class Alloc, class Release>
+inline bool adj_alloc_reverse(AdjointState* A, size_t N, Alloc alloc, Release release) {
+  if (A->reverse) return true;
+  const size_t K1 = (size_t)A->K + 1;
+  A->reverse = adj_alloc_all(
+      A,
+      {{(void**)&A->abar[0], 19 * N * 8}, {(void**)&A->abar[1], 19 * N * 8}, {(void**)&A->P, 19 * N * 8},
+       {(void**)&A->mbar[0], N * 8}, {(void**)&A->mbar[1], N * 8}, {(void**)&A->phibar[0], N * 8},
+       {(void**)&A->phibar[1], N * 8}, {(void**)&A->theta, 64}, {(void**)&A->dphi0, N * 8},
+       {&A->seg_f, A->fbytes * K1}, {(void**)&A->seg_m, N * 8 * K1}, {&A->seg_phi, A->rbytes * K1},
+       {(void**)&A->seg_flags, N * K1}, {(void**)&A->Mh, N * 8}, {(void**)&A->flist, 2 * (2 * N + 2) * sizeof(int)},
+       {(void**)&A->rh, N * 8}, {(void**)&A->ngb, N * 4 * 8}},
+      alloc, release);
+  return A->reverse;
+}
 
 // blocks of the objective's reduction, and the doubles of AdjointState::red:
 // result, count, a block counter, then two partial sums per block
