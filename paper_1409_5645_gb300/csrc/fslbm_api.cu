@@ -556,7 +556,7 @@ static int step_t(fslbm* h) {
   }
   if (mark_event(h, 3)) return 1;
   if (!h->par.freeze) {
-    int rc = launch_conversions<P>(h->par, v, h->st, h->list_blocks, h->coop_blocks, mr);
+    int rc = launch_conversions<P>(par, v, h->st, h->list_blocks, h->coop_blocks, mr);
     if (rc == (int)cudaErrorCooperativeLaunchTooLarge && h->coop_blocks > 0) {
       // the device cannot hold the cooperative grid now (e.g. shared with
       // other work): four launches and the stand-alone reduction from here on
@@ -565,7 +565,7 @@ static int step_t(fslbm* h) {
       fslbm_drop_graphs(h);
       if (mr.nb > 0 && launch_reduce(h->partials, nparts, h->red, h->red_blocks, h->lost, h->step_mass, h->st))
         return 1;
-      rc = launch_conversions<P>(h->par, v, h->st, h->list_blocks, 0, MassReduce{});
+      rc = launch_conversions<P>(par, v, h->st, h->list_blocks, 0, MassReduce{});
     }
     if (rc) return 1;
   }
