@@ -15,6 +15,7 @@
 
 #include "fslbm.h"
 #include "fslbm_dev.cuh"
+#include "fslbm_fixed.cuh"
 #include "fslbm_handle.h"
 #include "fslbm_kernels.h"
 
@@ -187,22 +188,7 @@ extern "C" int fslbm_create_ex(const fslbm_params* prm, fslbm_t** out) {
   p.elvira = q.elvira;
   p.adj32 = q.adjoint_fp32 && q.precision != FSLBM_F64;
   p.umax2 = q.u_max * q.u_max;
-  {
-    // the FP64 form's collision in fixed point: |lambda| < 2 holds for every
-    // tau > 1/2; the forces must leave the operands in range
-    bool ok = !p.compressible && !p.linear_eq;
-    for (int a = 0; a < 3; ++a) {
-      const double gl = p.g[a] * p.inv_lam_m;
-      ok = ok && fabs(p.g[a]) < 1.0 / 32.0 && fabs(gl) < 1.0 / 8.0;
-      p.fx_hg[a] = ok ? llround(p.g[a] * 0x1p59) : 0;
-      p.fx_gl[a] = ok ? llround(gl * 0x1p60) : 0;
-    }
-    ok = ok && p.lam_p > -2.0 && p.lam_p < 0.0 && p.lam_m > -2.0 && p.lam_m < 0.0;
-    p.fx_lp = ok ? llround(p.lam_p * 0x1p62) : 0;
-    p.fx_lm = ok ? llround(p.lam_m * 0x1p62) : 0;
-    p.fx_um2 = p.umax2 > 0.0 && p.umax2 < 4.0 ? llround(p.umax2 * 0x1p60) : 0x7fffffffffffffffLL;
-    p.fix_ok = ok;
-  }
+  fix_constants(p);
 
   const size_t Nn = (size_t)N, N4 = (Nn + 3) & ~(size_t)3;
   h->cap = (int)N;

@@ -169,6 +169,7 @@ struct Par {
   long long fx_lp, fx_lm;  // lambda_+-, units of 2^-62
   long long fx_hg[3];      // g / 2, units of 2^-60
   long long fx_gl[3];      // g / lambda_-
+  long long fx_gm[3];      // what its rounding leaves, / 3, units of 2^-91 (see FixTerms)
   long long fx_um2;        // u_max^2 (the largest value: off)
 #ifdef FSLBM_CHECKED
   int* err;                // the handle's error word (bounds-checked build)
