@@ -19,9 +19,9 @@
 // FP64 run's by 1e-15 of its value a step.
 //
 // A cell whose populations are not all in [0, 1/4) (rest: [0, 1)), whose
-// density reaches 2 or its momentum 1/2, or whose result leaves [2^-28, 8) takes
-// collide<double> (or, for the last, the hardware conversion): negative
-// populations, NaN and states far from rho = 1 included.  Values below 2^-8
+// density is not in [1/2, 2), whose momentum reaches 1/2, or whose result
+// leaves [2^-28, 8) takes collide<double> (or, for the last, the hardware
+// conversion): negative populations, NaN and states far from rho = 1 included.  Values below 2^-8
 // are rounded to the unit, which FP64's own sums with their neighbours do too.
 #pragma once
 #include <math.h>
@@ -133,10 +133,14 @@ inline void fix_constants(Par& p) {
   p.fix_ok = ok;
 }
 
-// density below 2 (4 rho fits), |j| < 1/2 (with the populations' range, every product below)
+// Density in [1/2, 2), |j| < 1/2.  With the populations' range the upper bounds
+// keep every product below (4 rho fits).  The lower one is for the unit, which
+// is absolute: at a density of 1/2 FP64's own chain still errs twice as far (8e-18
+// rms), below 1/4 it is the nearer one, and a density of zero has to reach its
+// check there.
 __host__ __device__ __forceinline__ bool fix_range(long long r, long long jx, long long jy, long long jz) {
   auto half = [](long long j) { return (unsigned)((int)(j >> 32) + 0x08000000) < 0x10000000u; };
-  return (unsigned)(r >> 32) < 0x20000000u && half(jx) && half(jy) && half(jz);
+  return (unsigned)((int)(r >> 32) - 0x08000000) < 0x18000000u && half(jx) && half(jy) && half(jz);
 }
 
 // What a cell's populations share, and the collision of the rest population
