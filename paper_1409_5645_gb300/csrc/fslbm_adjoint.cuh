@@ -163,7 +163,7 @@ __device__ __forceinline__ void collide_rev64(const Par& p, const double (&f)[19
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
     ub[a] += 3.0 * nl * dens * u[a];
-    th[2 + a] += 0.5 * ub[a] - vb[a] * p.inv_lam_m;
+    th[2 + a] += 0.5 * ub[a] - quot_near(vb[a], lm, p.inv_lam_m);
     ub[a] += vb[a];
   }
   th[1] += (g0 * vb[0] + g1 * vb[1] + g2 * vb[2]) / (lm * lm);

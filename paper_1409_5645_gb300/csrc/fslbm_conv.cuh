@@ -164,8 +164,11 @@ __device__ __forceinline__ void newg_cell(const Par& p, const View<P>& v, int k)
     // (rbar is rho - 1 in the shifted forms: the mean of rho - 1)
     R rbar, u0, u1, u2;
     if constexpr (P == P64) {  // (one FP64 division for four: they bound the FP64 form's stage)
-      const R ic = R(1) / R(c);
-      rbar = rs * ic; u0 = s0 * ic; u1 = s1 * ic; u2 = s2 * ic;
+      const R dc = R(c), ic = R(1) / dc;
+      rbar = quot_near(rs, dc, ic);
+      u0 = quot_near(s0, dc, ic);
+      u1 = quot_near(s1, dc, ic);
+      u2 = quot_near(s2, dc, ic);
     } else {
       rbar = rs / R(c); u0 = s0 / R(c); u1 = s1 / R(c); u2 = s2 / R(c);
     }

@@ -354,6 +354,15 @@ __device__ __forceinline__ double fx_add(double a, double b) { return __dadd_rn(
 __device__ __forceinline__ float fx_sub(float a, float b) { return __fsub_rn(a, b); }
 __device__ __forceinline__ double fx_sub(double a, double b) { return __dsub_rn(a, b); }
 
+// a / b to the nearest from ib, the FP64 value nearest to 1 / b: the product and
+// its exact remainder (Markstein, "Computation of elementary functions on the
+// IBM RISC System/6000 processor", IBM J. Res. Dev. 34, 1990).  Several
+// quotients of one divisor cost one division.
+__host__ __device__ __forceinline__ double quot_near(double a, double b, double ib) {
+  const double q = a * ib;
+  return fma(fma(-b, q, a), ib, q);
+}
+
 // c.u for a lattice direction (components 0 or +-1: exact adds)
 template <class R, int q>
 __device__ __forceinline__ R cdot(R ux, R uy, R uz) {
@@ -647,7 +656,7 @@ __device__ R plic_offset(R nx_, R ny_, R nz_, R ph) {
   R L1 = a0 + a1 + a2;
   if constexpr (sizeof(R) == 8) {  // (one FP64 division for three)
     const R il = R(1) / L1;
-    a0 *= il; a1 *= il; a2 *= il;
+    a0 = quot_near(a0, L1, il); a1 = quot_near(a1, L1, il); a2 = quot_near(a2, L1, il);
   } else {
     a0 /= L1; a1 /= L1; a2 /= L1;
   }
@@ -908,8 +917,8 @@ __device__ __forceinline__ void geometry_finish(const Par& p, const uint8_t* __r
       const R il = rsqrtf(v0 * v0 + v1 * v1 + v2 * v2);
       n[0] = v0 * il; n[1] = v1 * il; n[2] = v2 * il;
     } else {
-      const R il = R(1) / sqrt(v0 * v0 + v1 * v1 + v2 * v2);
-      n[0] = v0 * il; n[1] = v1 * il; n[2] = v2 * il;
+      const R len = sqrt(v0 * v0 + v1 * v1 + v2 * v2), il = R(1) / len;
+      n[0] = quot_near(v0, len, il); n[1] = quot_near(v1, len, il); n[2] = quot_near(v2, len, il);
     }
     R nabs = fabs(a == 0 ? n[0] : (a == 1 ? n[1] : n[2]));
     d = nabs * (H[4] - R(3.5));
@@ -933,8 +942,8 @@ __device__ __forceinline__ void geometry_finish(const Par& p, const uint8_t* __r
       const R il = rsqrtf(nn);
       n[0] *= il; n[1] *= il; n[2] *= il;
     } else {
-      const R il = R(1) / sqrt(nn);
-      n[0] *= il; n[1] *= il; n[2] *= il;
+      const R len = sqrt(nn), il = R(1) / len;
+      n[0] = quot_near(n[0], len, il); n[1] = quot_near(n[1], len, il); n[2] = quot_near(n[2], len, il);
     }
     d = plic_offset<R>(n[0], n[1], n[2], phic);
   }
