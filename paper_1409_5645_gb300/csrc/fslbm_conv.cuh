@@ -69,25 +69,25 @@ __device__ __forceinline__ void fill_cell(const Par& p, const View<P>& v, int k)
     push(won, v.nglist, &v.cnt[3], v.cap, (int)j, v.err);
   }
 }
-// The FP64 form's new cell from its neighbours' fixed-point moments (rho, j;
-// lanes with `use`): f^eq of the means, collided; lane q builds population q.
-// Its density and momentum are the means themselves (the weights' sums), as a
-// sum over the lanes would give them back up to rounding.
+// The FP64 form's new cell from its neighbours' fixed-point moments (rho - 1,
+// j; lanes with `use`): f^eq of the means, collided; lane q builds population q.
+// The sums are exact (moments_fixed).  The cell's density and momentum are the
+// means themselves (the weights' sums), as a sum over the lanes would give
+// them back up to rounding.
 __device__ __forceinline__ void newg_fixed(const Par& p, const View<P64>& v, long long j, int q, bool use,
-                                           long long xr, const long long (&xj)[3]) {
+                                           long long dev, const long long (&xj)[3]) {
   const unsigned FULL = 0xffffffffu;
   const int lane = threadIdx.x & 31;
-  // (shifted so that 18 of them stay in range)
-  long long m[4] = {use ? xr >> 5 : 0, use ? xj[0] >> 3 : 0, use ? xj[1] >> 3 : 0, use ? xj[2] >> 3 : 0};
-  const int c = __popc(__ballot_sync(FULL, use));
+  long long m[4] = {use ? dev : 0, use ? xj[0] : 0, use ? xj[1] : 0, use ? xj[2] : 0};
+  const double c = (double)__popc(__ballot_sync(FULL, use)), ic = 1.0 / c;
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1)
 #pragma unroll
     for (int k = 0; k < 4; ++k) m[k] += __shfl_xor_sync(FULL, m[k], o);
-  const double ic = 1.0 / (double)c;
-  const double rho = double_of_fix(m[0]) * 32.0 * ic;
-  const double u0 = double_of_fix(m[1]) * 8.0 * ic - 0.5 * p.g[0], u1 = double_of_fix(m[2]) * 8.0 * ic - 0.5 * p.g[1],
-               u2 = double_of_fix(m[3]) * 8.0 * ic - 0.5 * p.g[2];
+  const double rho = 1.0 + quot_near(double_of_fix(m[0]), c, ic);
+  const double u0 = quot_near(double_of_fix(m[1]), c, ic) - 0.5 * p.g[0],
+               u1 = quot_near(double_of_fix(m[2]), c, ic) - 0.5 * p.g[1],
+               u2 = quot_near(double_of_fix(m[3]), c, ic) - 0.5 * p.g[2];
   const double w = q == 0 ? 1.0 / 3.0 : (q <= 6 ? 1.0 / 18.0 : 1.0 / 36.0);
   const double ax = cx(q), ay = cy(q), az = cz(q);
   const double cu = ax * u0 + ay * u1 + az * u2, usq = u0 * u0 + u1 * u1 + u2 * u2;
@@ -119,7 +119,7 @@ __device__ __forceinline__ void newg_cell(const Par& p, const View<P>& v, int k)
     coords(p, j, x, y, z);
     bool use = false, range = true;
     R rr = R(0), ux = R(0), uy = R(0), uz = R(0);
-    long long xr = 0, xj[3] = {0, 0, 0};  // the neighbour's moments in fixed point (FP64 form)
+    long long xr = 0, xj[3] = {0, 0, 0};  // the neighbour's rho - 1 and j in fixed point (FP64 form)
     if (lane >= 1 && lane < 19) {
       long long y2 = nbr(p, x, y, z, cx(q), cy(q), cz(q));
       if (y2 >= 0) {
@@ -146,7 +146,7 @@ __device__ __forceinline__ void newg_cell(const Par& p, const View<P>& v, int k)
         return;
       }
       if (use && range) {
-        rr = double_of_fix(xr);
+        rr = 1.0 + double_of_fix(xr);
         ux = double_of_fix(xj[0]) - 0.5 * p.g[0];
         uy = double_of_fix(xj[1]) - 0.5 * p.g[1];
         uz = double_of_fix(xj[2]) - 0.5 * p.g[2];

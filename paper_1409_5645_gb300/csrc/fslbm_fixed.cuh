@@ -302,24 +302,26 @@ __device__ __forceinline__ bool collide_warp(const Par& p, int q, double& f, lon
 }
 #endif
 
-// density and momentum of populations in the collision's range, in units of
-// 2^-60; false where they are not
-__host__ __device__ __forceinline__ bool moments_fixed(const double (&f)[19], long long& rho, long long (&j)[3]) {
+// Density less 1 and momentum of populations in the collision's range, in units
+// of 2^-60; false where they are not, or where one of the four reaches 7/16
+// (so that eighteen cells' sum fits 64 bits)
+__host__ __device__ __forceinline__ bool moments_fixed(const double (&f)[19], long long& dev, long long (&j)[3]) {
   bool in = (unsigned)(bits_of_double(f[0]) >> 32) < FIX_REST;
 #pragma unroll
   for (int q = 1; q < 19; ++q) in = in && (unsigned)(bits_of_double(f[q]) >> 32) < FIX_MOVING;
   if (!in) return false;
-  rho = fix_near(bits_of_double(f[0]));
+  dev = fix_near(bits_of_double(f[0])) - (1LL << 60);
   j[0] = j[1] = j[2] = 0;
 #pragma unroll
   for (int q = 1; q < 19; q += 2) {
     const long long a = fix_near(bits_of_double(f[q])), b = fix_near(bits_of_double(f[q + 1]));
-    rho += a + b;
+    dev += a + b;
     j[0] += cx(q) * (a - b);
     j[1] += cy(q) * (a - b);
     j[2] += cz(q) * (a - b);
   }
-  return true;
+  auto small = [](long long v) { return (unsigned)((int)(v >> 32) + 0x07000000) < 0x0e000000u; };
+  return small(dev) && small(j[0]) && small(j[1]) && small(j[2]);
 }
 
 }  // namespace fsl
