@@ -237,8 +237,13 @@ int fslbm_set_state_post(fslbm_t *h, const uint8_t *flags, const double *f_post,
 /* Advance n >= 0 time steps.  Asynchronous on the handle's stream: returns
  * launch errors only; method faults appear at the next synchronising call.
  * One call of n steps gives the bits of n calls of one step and costs less
- * host time (steps go out as CUDA graphs, or many in one launch on a small
- * lattice; the graphs belong to the handle). */
+ * host time: steps go out as CUDA graphs (which belong to the handle), and a
+ * call of more than four steps of a lattice of up to 65 536 cells without the
+ * shear term, u_b extrapolation, normal links, ELVIRA or, in FP64, another
+ * equilibrium than the default (fslbm_params) takes all but its last step in
+ * one launch of another kernel, which has its own loads (bulk_loads names
+ * those of the step's kernels).  Not so while fslbm_timing is on, on a
+ * capturing stream, or after fslbm_set_overlap(h, 0). */
 int fslbm_step(fslbm_t *h, int n);
 
 /* Wait for the handle's stream; return the sticky device error, if any. */
@@ -390,26 +395,30 @@ int fslbm_halo_unpack(fslbm_t *h, const int lo[3], const int hi[3], const void *
 /* Steps taken since the last set_state. */
 long long fslbm_time(const fslbm_t *h);
 
-/* The fslbm_loads the bulk kernel of this handle uses (FSLBM_ERR_ARG for
- * NULL).  An implementation property with no counterpart in the paper. */
+/* The fslbm_loads the bulk kernel of this handle uses where steps go by the
+ * step's kernels (FSLBM_ERR_ARG for NULL).  An implementation property with no
+ * counterpart in the paper. */
 int fslbm_bulk_loads(const fslbm_t *h);
 
 /* Scheduling of the interface kernels (an implementation choice with no
  * counterpart in the paper; the results are the same either way, bit for
  * bit).  on = 1 (default): after the segment scan the interface geometry,
- * and beside the two-cells-per-lane bulk kernel the interface kernel too,
- * run on a second stream of the handle while the bulk kernel runs on its
- * stream; the pair kernel's grid then leaves room for them on every SM, and
- * the streams join before the conversions.  on = 0: every kernel in order on
- * the handle's stream, the bulk kernel on a full resident wave (to time the
- * kernels alone).  FSLBM_ERR_ARG for other values. */
+ * and beside the two-cells-per-lane bulk kernel and the FP64 one the interface
+ * kernel too, run on a second stream of the handle while the bulk kernel runs
+ * on its stream; the pair kernel's grid then leaves room for them on every SM,
+ * and the streams join before the conversions; a call of more than four steps
+ * of a small lattice (see fslbm_step) takes all but the last in one launch.
+ * on = 0: every kernel of every step in order on the handle's stream, the bulk
+ * kernel on a full resident wave (to time the kernels alone).  FSLBM_ERR_ARG
+ * for other values. */
 int fslbm_set_overlap(fslbm_t *h, int on);
 
-/* Kernel launches one fslbm_step time step makes on this handle (the
- * per-step reset, segment list, bulk, interface geometry where the rule,
- * surface tension, the shear term or the normal links need it, interface,
- * the two-level mass reduction, and the conversions: one cooperative launch
- * where the device allows it, else four; none with frozen flags), or
+/* Kernel launches of one time step by the step's kernels on this handle, one
+ * by one or in a graph; a small lattice's longer calls take fewer (fslbm_step).
+ * They are the per-step reset, segment list, bulk, interface geometry where the
+ * rule, surface tension, the shear term or the normal links need it,
+ * interface, the two-level mass reduction, and the conversions: one cooperative
+ * launch where the device allows it, else four; none with frozen flags.
  * FSLBM_ERR_ARG for NULL.  An implementation property with no counterpart in
  * the paper. */
 int fslbm_launches_per_step(const fslbm_t *h);

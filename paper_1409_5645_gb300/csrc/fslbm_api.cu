@@ -675,7 +675,7 @@ static bool small_steps(fslbm* h, int steps, const StateLog& log) {
   return true;
 }
 
-// the handle's stream takes whole graphs and many-steps launches now
+// the handle's stream takes whole graphs (and many-steps launches) now
 static bool whole_steps(fslbm* h) {
   if (h->graph_off || h->timing) return false;
   cudaStreamCaptureStatus s = cudaStreamCaptureStatusNone;
@@ -686,10 +686,14 @@ static bool whole_steps(fslbm* h) {
   return s == cudaStreamCaptureStatusNone;
 }
 
+// The many-steps launch, where the step's kernels are not asked for in order
+// (fslbm_set_overlap)
+static bool many_steps(const fslbm* h) { return h->small_blocks > 0 && h->overlap; }
+
 // n steps of a small lattice in one launch, the state after step k (1 .. n) at
 // slot k of the log; false: not done
 bool fslbm_logged_steps(fslbm* h, int n, const StateLog& log) {
-  if (n < 1 || h->small_blocks <= 0 || !whole_steps(h) || !small_steps(h, n, log)) return false;
+  if (n < 1 || !many_steps(h) || !whole_steps(h) || !small_steps(h, n, log)) return false;
   h->t += n;
   return true;
 }
@@ -699,8 +703,9 @@ extern "C" int fslbm_step(fslbm_t* h, int n) {
   bool graphs = whole_steps(h);
   int s0 = 0;
   // a small lattice: all but the last step in launches of up to SMALL_STEPS
+  // (a call of up to SMALL_LEAST steps goes by the step's kernels)
   constexpr int SMALL_STEPS = 256, SMALL_LEAST = 4;
-  while (graphs && h->small_blocks > 0 && n - s0 > SMALL_LEAST) {
+  while (graphs && many_steps(h) && n - s0 > SMALL_LEAST) {
     const int k = n - s0 - 1 < SMALL_STEPS ? n - s0 - 1 : SMALL_STEPS;
     if (!small_steps(h, k, StateLog{})) break;
     s0 += k;

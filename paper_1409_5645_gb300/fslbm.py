@@ -410,13 +410,14 @@ class Lattice:
         return {v: k for k, v in LOADS.items()}[self.L.fslbm_bulk_loads(self.h)]
 
     def set_overlap(self, on: bool):
-        """Interface kernels on a second stream beside the bulk kernel (True,
-        the default) or every kernel in order on the handle's stream."""
+        """Interface kernels on a second stream beside the bulk kernel, and many
+        steps of a small lattice in one launch (True, the default), or every
+        kernel in order on the handle's stream."""
         self._check(self.L.fslbm_set_overlap(self.h, int(bool(on))), "set_overlap")
 
     @property
     def launches_per_step(self) -> int:
-        """Kernel launches one time step makes on this lattice."""
+        """Kernel launches of one time step by the step's kernels on this lattice."""
         return int(self.L.fslbm_launches_per_step(self.h))
 
     @property
