@@ -305,8 +305,9 @@ enum fslbm_objective {
  * checkpoint (flags, f~, m, phi) every K >= 1 steps, and return J.  Holds
  * ceil(nsteps/K) checkpoints on the device until the handle's state is set
  * again or the handle is destroyed; device buffers of up to 2 GiB in all stay
- * with the handle after a new state, for the next differentiation with the
- * same K and number of checkpoints. */
+ * with the handle after a new state, for a next differentiation with the same K
+ * and number of checkpoints, and go with the new state after that (or when the
+ * handle finds no memory for something else). */
 int fslbm_adjoint_forward(fslbm_t *h, int nsteps, int K, int objective, double *J);
 
 /* Reverse pass (once per forward pass): recompute each K-step segment from

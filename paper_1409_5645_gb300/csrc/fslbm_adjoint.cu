@@ -108,15 +108,22 @@ void fslbm_free_adjoint(fslbm* h) {
 // A new state ends a differentiation.  Its buffers (some twenty allocations,
 // up to ADJ_KEEP_BYTES) stay with the handle for the next one of the same
 // window: allocating and freeing them was most of a short differentiation of a
-// 128x64x64 lattice.  Larger ones are given back at once.
+// 128x64x64 lattice.  Larger ones are given back at once, and those that are
+// not used before one more new state with that one, or when the handle finds no
+// memory for something else.
 constexpr size_t ADJ_KEEP_BYTES = (size_t)2 << 30;
 void fslbm_end_adjoint(fslbm* h) {
   if (!h->adj) return;
-  if (h->adj->bytes > ADJ_KEEP_BYTES) {
+  if (h->adj->bytes > ADJ_KEEP_BYTES || !h->adj->live) {
     fslbm_free_adjoint(h);
     return;
   }
   h->adj->ready = h->adj->live = false;
+}
+bool fslbm_yield_adjoint(fslbm* h) {
+  if (!h->adj || h->adj->live) return false;
+  fslbm_free_adjoint(h);
+  return true;
 }
 
 static bool amalloc(void** p, size_t bytes) {

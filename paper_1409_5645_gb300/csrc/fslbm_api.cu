@@ -88,12 +88,19 @@ static void free_all(fslbm* h) {
   h->tmap = nullptr;
 }
 
+// device memory for the handle; the buffers that an ended differentiation left
+// (fslbm_end_adjoint) go before it is refused
+static bool device_alloc(fslbm* h, void** p, size_t bytes) {
+  do {
+    if (cudaMalloc(p, bytes ? bytes : 16) == cudaSuccess) return true;
+    cudaGetLastError();  // (reported by the caller; the next launch must not find it)
+  } while (fslbm_yield_adjoint(h));
+  *p = nullptr;
+  return false;
+}
 template <class T>
 static bool dalloc(fslbm* h, T** p, size_t bytes) {
-  if (cudaMalloc((void**)p, bytes ? bytes : 16) != cudaSuccess) {
-    *p = nullptr;
-    return false;
-  }
+  if (!device_alloc(h, (void**)p, bytes)) return false;
   h->bytes += bytes;
   return true;
 }
@@ -374,7 +381,7 @@ static int stage(fslbm* h, const void* src, size_t bytes, int where, Staged& s) 
     s.dev = src;
     return FSLBM_OK;
   }
-  CK(cudaMalloc(&s.owned, bytes), "cudaMalloc (staging)");
+  if (!device_alloc(h, &s.owned, bytes)) return fail(h, FSLBM_ERR_CUDA, "cudaMalloc (staging)", cudaErrorMemoryAllocation);
   CK(cudaMemcpyAsync(s.owned, src, bytes, cudaMemcpyHostToDevice, h->st), "H2D copy");
   s.dev = s.owned;
   return FSLBM_OK;
@@ -750,7 +757,7 @@ extern "C" int fslbm_get_fields(fslbm_t* h, unsigned mask, void* const* out, int
     if (!out[k]) return fail(h, FSLBM_ERR_ARG, "NULL output buffer");
     if (where == FSLBM_DEVICE) {
       dev[k] = out[k];
-    } else if (cudaMalloc(&owned[k], sizes[b]) != cudaSuccess) {
+    } else if (!device_alloc(h, &owned[k], sizes[b])) {
       rc = fail(h, FSLBM_ERR_OOM, "staging allocation");
       break;
     } else {

@@ -14,6 +14,8 @@ struct fslbm;
 void fslbm_free_adjoint(fslbm* h);
 // a new state ends a differentiation (fslbm_adjoint.cu): its buffers stay up to a limit
 void fslbm_end_adjoint(fslbm* h);
+// give back the buffers that an ended differentiation left; false: there are none
+bool fslbm_yield_adjoint(fslbm* h);
 
 struct fslbm {
   fslbm_params prm;
