@@ -18,7 +18,7 @@ constexpr int BULK64_BLOCKS = 4;  // resident blocks of 128 threads per SM
 
 __global__ void __launch_bounds__(128, BULK64_BLOCKS) k_bulk_fixed(Par p, View<P64> v,
                                                                    const int* __restrict__ seglist,
-                                                                   const int* __restrict__ segcount, int nparts) {
+                                                                   const int* __restrict__ segcount) {
   pdl_begin();
   const int nseg = *((volatile const int*)segcount);
   const int lane = threadIdx.x & 31;
@@ -95,13 +95,11 @@ __global__ void __launch_bounds__(128, BULK64_BLOCKS) k_bulk_fixed(Par p, View<P
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) msum += __shfl_down_sync(0xffffffffu, msum, o);
   if (lane == 0) v.partials[gw] = msum;
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (nw + t < nparts) v.partials[nw + t] = 0.0;
 }
 
 int launch_bulk_fixed(const Par& p, const View<P64>& v, cudaStream_t st, int bulk_blocks, const int* seglist,
                       const int* segcount) {
-  return launch_k(k_bulk_fixed, bulk_blocks, 128, 0, st, p, v, seglist, segcount, bulk_blocks * 4);
+  return launch_k(k_bulk_fixed, bulk_blocks, 128, 0, st, p, v, seglist, segcount);
 }
 
 }  // namespace fsl

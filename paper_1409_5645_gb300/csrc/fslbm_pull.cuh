@@ -32,7 +32,7 @@ __device__ __forceinline__ void warp_append(bool pred, int value, int* list, int
 template <int P, bool IN = false>
 __device__ __forceinline__ void pull_general(const Par& p, const View<P>& v, int x, int y, int z,
                                              typename Form<P>::R (&f)[19], unsigned& wallm, unsigned& gasm,
-                                             unsigned* liqm = nullptr, int* srcs = nullptr) {
+                                             unsigned* liqm = nullptr) {
   const size_t N = (size_t)p.N;
   wallm = 0u;
   gasm = 0u;
@@ -72,7 +72,6 @@ __device__ __forceinline__ void pull_general(const Par& p, const View<P>& v, int
         s = nbr(p, x, y, z, -cx(q), -cy(q), -cz(q));
       }
       uint8_t ks = kind_at(v.flags, s);
-      if (srcs) srcs[q] = (int)s;
       if (is_fluid(ks)) {
         f[q] = ldq<P>(v.fin, (size_t)q * N + (size_t)s, q);
         if (ks == LIQ) lm |= 1u << q;
