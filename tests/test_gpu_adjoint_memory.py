@@ -26,8 +26,13 @@ def test_buffers_are_kept_for_one_state_and_given_back():
         J = g.adjoint_forward(6, 3)
         return J, *g.adjoint_backward()
 
-    for _ in range(20):  # (graphs and streams of the handle are made)
+    # the handle's graphs, and what the driver keeps for kernels once they have run
+    for _ in range(20):
         g.step(8)
+    other = fslbm.Lattice.from_case(c, precision="f32", keep_f0=1)
+    other.adjoint_forward(6, 3)
+    other.adjoint_backward()
+    other.close()
     state()
     before, mib = free(), 2 ** 20
     first = gradient()
