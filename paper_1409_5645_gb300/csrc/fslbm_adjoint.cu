@@ -172,7 +172,7 @@ extern "C" int fslbm_adjoint_forward(fslbm_t* h, int nsteps, int K, int objectiv
   }
   AdjointState* A = h->adj;
   const size_t N = (size_t)h->par.N;
-  A->nsteps = nsteps;
+  A->nsteps = h->window = nsteps;
   A->K = K;
   A->objective = objective;
   A->nck = nck;

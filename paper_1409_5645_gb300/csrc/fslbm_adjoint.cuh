@@ -435,8 +435,8 @@ __global__ void __launch_bounds__(128) k_adj_local(Par p, AdjView<P> a) {
           unsigned st[3] = {0u, 0u, 0u};
           R nn, kopen;
           const bool ok = coop_stencil<R, false>(p, a.flags, a.phi, xk, yk, zk, in3, (int)ik, ph, nn, kopen, G, st);
+          if (ok) coop_finish<R, false, false>(p, a.flags, a.phi, xk, yk, zk, ph, nn, kopen, G);
           if (lane == 0) {
-            if (ok) geometry_finish<R, false, false>(p, a.flags, a.phi, xk, yk, zk, ph, nn, &kopen, G);
             wgeo[k].G = G;
             wgeo[k].stored[0] = st[0]; wgeo[k].stored[1] = st[1]; wgeo[k].stored[2] = st[2];
           }

@@ -619,17 +619,20 @@ static int enqueue_step(fslbm* h) {
 // graphs belong to the handle: captured on a stream of its own at the first
 // use, dropped when a parameter they hold changes.  A call whose stream is
 // itself being captured, a timed step and a device that refuses a capture take
-// the kernels one by one, and so do a handle's first GRAPH_AFTER steps: an
-// eight-step graph costs 60 to 110 us to make, a single-step one 35 us, and a
-// step saves 5 to 15 us by them.  (A fresh handle, us, graphs from the first
-// step -> from the seventeenth: step(8) of 128x64x64 FP32 743 -> 628, FP64 1138
-// -> 1025, of 256x128x128 FP64 1817 -> 1677; step(40) 2395 -> 2352, 4337 ->
-// 4274, 7520 -> 7414; forty steps all by kernels with a timed step's events:
-// 2841, 4533, 7533.)
+// the kernels one by one, and so do steps for which no graph is there yet, of a
+// call with fewer than GRAPH_CALL to go by kernels (in a differentiation, of a
+// window of fewer), while the handle has had fewer than GRAPH_CALL such steps
+// (for a single-step graph: GRAPH_SINGLE): an eight-step graph costs 60 to
+// 110 us to make, a single-step one 35 us, and a step saves 5 to 15 us by the
+// one, up to 45 us by the other.  (A fresh handle, us, by graphs / by kernels:
+// step(8) of 128x64x64 FP32 743 / 628, FP64 1138 / 1025, of 256x128x128 FP64 1817 /
+// 1677; step(16) 1153 / 1087, 1919 / 1856, 3167 / 3028; step(24) 1596 / 1800 with a
+// timed step's events, 2770 / 2797, 4635 / 4560; once, twice and four times step(1)
+// of 24x8x16 FP64 126 / 91, 186 / 175, 308 / 322.)
 // Measured (GB300, us per step, kernel by kernel -> graphs): 4x4x32 FP64 film
 // 89.1 -> 82.0, 128x64x64 FP32 splash 110.4 -> 102.7, 512x256x256 FP32 506 ->
 // 499; the shorter a step's kernels are, the more of it the launches were.
-constexpr int GRAPH_STEPS = 8, GRAPH_AFTER = 16;
+constexpr int GRAPH_STEPS = 8, GRAPH_CALL = 16, GRAPH_SINGLE = 2;
 
 static cudaGraphExec_t capture_steps(fslbm* h, int steps) {
   if (!h->capture && cudaStreamCreateWithFlags(&h->capture, cudaStreamNonBlocking) != cudaSuccess) {
@@ -727,7 +730,10 @@ extern "C" int fslbm_step(fslbm_t* h, int n) {
   for (int s = s0; s < n;) {
     const int k = n - s >= GRAPH_STEPS ? GRAPH_STEPS : 1;
     graphs = graphs && !h->graph_off;
-    if (graphs && h->plain_steps >= GRAPH_AFTER && graph_steps(h, k)) {
+    const bool worth = h->graph[h->fp64_chain][h->cur][k > 1] ||
+                       (h->fp64_chain ? h->window : n - s0) >= GRAPH_CALL ||
+                       h->plain_steps >= (k > 1 ? GRAPH_CALL : GRAPH_SINGLE);
+    if (graphs && worth && graph_steps(h, k)) {
       s += k;
       h->t += k;
       continue;
@@ -735,7 +741,7 @@ extern "C" int fslbm_step(fslbm_t* h, int n) {
     if (enqueue_step(h)) return fail(h, FSLBM_ERR_CUDA, "step launch", cudaGetLastError());
     s += 1;
     h->t += 1;
-    if (h->plain_steps < GRAPH_AFTER) h->plain_steps += 1;
+    if (h->plain_steps < GRAPH_CALL) h->plain_steps += 1;
   }
   return FSLBM_OK;
 }

@@ -79,19 +79,21 @@ __device__ __forceinline__ void newg_fixed(const Par& p, const View<P64>& v, lon
   const unsigned FULL = 0xffffffffu;
   const int lane = threadIdx.x & 31;
   long long m[4] = {use ? dev : 0, use ? xj[0] : 0, use ? xj[1] : 0, use ? xj[2] : 0};
-  const double c = (double)__popc(__ballot_sync(FULL, use)), ic = 1.0 / c;
+  const int c = __popc(__ballot_sync(FULL, use));
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1)
 #pragma unroll
     for (int k = 0; k < 4; ++k) m[k] += __shfl_xor_sync(FULL, m[k], o);
-  const double rho = 1.0 + quot_near(double_of_fix(m[0]), c, ic);
-  const double u0 = quot_near(double_of_fix(m[1]), c, ic) - 0.5 * p.g[0],
-               u1 = quot_near(double_of_fix(m[2]), c, ic) - 0.5 * p.g[1],
-               u2 = quot_near(double_of_fix(m[3]), c, ic) - 0.5 * p.g[2];
+  // (a mean a lane: one FP64 division and conversion for the four)
+  const int l = lane & 3;
+  const double mean = double_of_fix(l == 0 ? m[0] : (l == 1 ? m[1] : (l == 2 ? m[2] : m[3]))) / (double)c;
+  const double rho = 1.0 + __shfl_sync(FULL, mean, 0);
+  const double u0 = __shfl_sync(FULL, mean, 1) - 0.5 * p.g[0], u1 = __shfl_sync(FULL, mean, 2) - 0.5 * p.g[1],
+               u2 = __shfl_sync(FULL, mean, 3) - 0.5 * p.g[2];
   const double w = q == 0 ? 1.0 / 3.0 : (q <= 6 ? 1.0 / 18.0 : 1.0 / 36.0);
   const double ax = cx(q), ay = cy(q), az = cz(q);
   const double cu = ax * u0 + ay * u1 + az * u2, usq = u0 * u0 + u1 * u1 + u2 * u2;
-  const double fp = w * (rho + 1.5 * (3.0 * cu * cu - usq)), fm = 3.0 * w * cu;  // even and odd part of f^eq
+  const double fp = w * rho + (w * 1.5) * (3.0 * cu * cu - usq), fm = 3.0 * w * cu;  // even and odd part of f^eq
   // the collision moves them toward e^+(u + g/2) and e^-(u - g/lambda_-)
   const double cg = ax * p.g[0] + ay * p.g[1] + az * p.g[2];
   const double ug = u0 * p.g[0] + u1 * p.g[1] + u2 * p.g[2], gg = p.g[0] * p.g[0] + p.g[1] * p.g[1] + p.g[2] * p.g[2];

@@ -354,13 +354,62 @@ __device__ __forceinline__ double fx_add(double a, double b) { return __dadd_rn(
 __device__ __forceinline__ float fx_sub(float a, float b) { return __fsub_rn(a, b); }
 __device__ __forceinline__ double fx_sub(double a, double b) { return __dsub_rn(a, b); }
 
-// a / b to the nearest from ib, the FP64 value nearest to 1 / b: the product and
-// its exact remainder (Markstein, "Computation of elementary functions on the
+// a / b to the nearest from ib, 1 / b to an ulp or so: the product and its exact
+// remainder (Markstein, "Computation of elementary functions on the
 // IBM RISC System/6000 processor", IBM J. Res. Dev. 34, 1990).  Several
 // quotients of one divisor cost one division.
 __host__ __device__ __forceinline__ double quot_near(double a, double b, double ib) {
   const double q = a * ib;
   return fma(fma(-b, q, a), ib, q);
+}
+
+// a0, a1, a2 divided by b.  WARP: a converged warp whose lanes hold the same
+// values, a lane per quotient: one division, without the products and
+// remainders
+template <bool WARP>
+__host__ __device__ __forceinline__ void quotients(double& a0, double& a1, double& a2, double b) {
+#ifdef __CUDA_ARCH__
+  if constexpr (WARP) {
+    const int l = threadIdx.x & 3;
+    const double q = (l == 0 ? a0 : (l == 1 ? a1 : a2)) / b;
+    a0 = __shfl_sync(0xffffffffu, q, 0);
+    a1 = __shfl_sync(0xffffffffu, q, 1);
+    a2 = __shfl_sync(0xffffffffu, q, 2);
+    return;
+  }
+#endif
+  const double ib = 1.0 / b;
+  a0 = quot_near(a0, b, ib);
+  a1 = quot_near(a1, b, ib);
+  a2 = quot_near(a2, b, ib);
+}
+// a0, a1, a2 divided by the square root of s > 0, root and quotients to the
+// nearest (as sqrt and a division give them): with y the reciprocal root (CUDA's
+// rsqrt, to an ulp or so), s y is the root but for half y times its remainder
+// s - (s y)^2, and the quotients are quot_near's.  WARP: a lane per component,
+// as quotients.  (A root and a division instead took 0.3 us more of a 4x4x32
+// film's 15 us step.)
+template <bool WARP>
+__host__ __device__ __forceinline__ void over_root(double& a0, double& a1, double& a2, double s) {
+#ifdef __CUDA_ARCH__
+  const double y = rsqrt(s);
+#else
+  const double y = 1.0 / sqrt(s);
+#endif
+  const double t = s * y, len = fma(fma(-t, t, s), 0.5 * y, t);
+#ifdef __CUDA_ARCH__
+  if constexpr (WARP) {
+    const int l = threadIdx.x & 3;
+    const double q = quot_near(l == 0 ? a0 : (l == 1 ? a1 : a2), len, y);
+    a0 = __shfl_sync(0xffffffffu, q, 0);
+    a1 = __shfl_sync(0xffffffffu, q, 1);
+    a2 = __shfl_sync(0xffffffffu, q, 2);
+    return;
+  }
+#endif
+  a0 = quot_near(a0, len, y);
+  a1 = quot_near(a1, len, y);
+  a2 = quot_near(a2, len, y);
 }
 
 // c.u for a lattice direction (components 0 or +-1: exact adds)
@@ -649,14 +698,13 @@ __host__ __device__ __forceinline__ double plic_alpha_polished(double tv, double
 // the side n.(x - x_c) <= d) of the plane cutting volume fraction ph.  The
 // fill is kept in [1e-9, 1 - 1e-9] first: at an empty or full corner the
 // inverse volume grows like a cube root and would turn rounding of ph into
-// visible plane shifts.
-template <class R>
+// visible plane shifts.  (WARP: see quotients)
+template <class R, bool WARP = false>
 __device__ R plic_offset(R nx_, R ny_, R nz_, R ph) {
   R a0 = fabs(nx_), a1 = fabs(ny_), a2 = fabs(nz_);
   R L1 = a0 + a1 + a2;
   if constexpr (sizeof(R) == 8) {  // (one FP64 division for three)
-    const R il = R(1) / L1;
-    a0 = quot_near(a0, L1, il); a1 = quot_near(a1, L1, il); a2 = quot_near(a2, L1, il);
+    quotients<WARP>(a0, a1, a2, L1);
   } else {
     a0 /= L1; a1 /= L1; a2 /= L1;
   }
@@ -898,7 +946,8 @@ __device__ __noinline__ void elvira_plane(const Par& p, const uint8_t* __restric
 // The normal, plane offset and curvature from the Parker-Youngs normal G.n
 // (not normalised, nn its square), the heights G.H and G.closed.  kopen: the
 // curvature where the columns are open, or NULL to have it computed here.
-template <class R, bool SIG, bool ELV>
+// WARP: called by a whole warp with the same values on every lane (coop_finish).
+template <class R, bool SIG, bool ELV, bool WARP = false>
 __device__ __forceinline__ void geometry_finish(const Par& p, const uint8_t* __restrict__ flags,
                                                 const R* __restrict__ phin, int x, int y, int z, R phic, R nn,
                                                 const R* kopen, Geo<R>& G) {
@@ -917,8 +966,8 @@ __device__ __forceinline__ void geometry_finish(const Par& p, const uint8_t* __r
       const R il = rsqrtf(v0 * v0 + v1 * v1 + v2 * v2);
       n[0] = v0 * il; n[1] = v1 * il; n[2] = v2 * il;
     } else {
-      const R len = sqrt(v0 * v0 + v1 * v1 + v2 * v2), il = R(1) / len;
-      n[0] = quot_near(v0, len, il); n[1] = quot_near(v1, len, il); n[2] = quot_near(v2, len, il);
+      n[0] = v0; n[1] = v1; n[2] = v2;
+      over_root<WARP>(n[0], n[1], n[2], v0 * v0 + v1 * v1 + v2 * v2);
     }
     R nabs = fabs(a == 0 ? n[0] : (a == 1 ? n[1] : n[2]));
     d = nabs * (H[4] - R(3.5));
@@ -942,10 +991,9 @@ __device__ __forceinline__ void geometry_finish(const Par& p, const uint8_t* __r
       const R il = rsqrtf(nn);
       n[0] *= il; n[1] *= il; n[2] *= il;
     } else {
-      const R len = sqrt(nn), il = R(1) / len;
-      n[0] = quot_near(n[0], len, il); n[1] = quot_near(n[1], len, il); n[2] = quot_near(n[2], len, il);
+      over_root<WARP>(n[0], n[1], n[2], nn);
     }
-    d = plic_offset<R>(n[0], n[1], n[2], phic);
+    d = plic_offset<R, WARP>(n[0], n[1], n[2], phic);
   }
 }
 
@@ -1234,6 +1282,15 @@ __device__ __forceinline__ bool coop_stencil(const Par& p, const uint8_t* __rest
   if (SIG && p.sigma != 0.0 && !G.closed)
     kopen = coop_curvature_open<R>(p, flags, phin, x, y, z, in3, i, G.n[0], G.n[1], G.n[2], a);
   return true;
+}
+
+// ... and the rest of it; the result is lane 0's
+template <class R, bool SIG, bool ELV>
+__device__ __forceinline__ void coop_finish(const Par& p, const uint8_t* __restrict__ flags,
+                                            const R* __restrict__ phin, int x, int y, int z, R phic, R nn, R kopen,
+                                            Geo<R>& G) {
+  constexpr bool WARP = sizeof(R) == 8 && !ELV;
+  if (WARP || (threadIdx.x & 31) == 0) geometry_finish<R, SIG, ELV, WARP>(p, flags, phin, x, y, z, phic, nn, &kopen, G);
 }
 
 // Fixed-order sum of chunk b of in[0, n) by the calling block of 256 threads:

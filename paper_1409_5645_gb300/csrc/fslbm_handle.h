@@ -65,7 +65,8 @@ struct fslbm {
   // steps captured as graphs (see fslbm_step): [fp64_chain][cur][0] one step, [..][1] GRAPH_STEPS steps
   cudaGraphExec_t graph[2][2][2];
   cudaStream_t capture;  // the capturing stream (created with the first graph), or NULL
-  int plain_steps;       // steps put out one kernel at a time, up to GRAPH_AFTER
+  int window;            // steps of the last differentiation's window
+  int plain_steps;       // steps put out one kernel at a time, up to GRAPH_CALL
   int graph_off;         // a capture or a graph launch failed: steps are launched one kernel at a time
 };
 

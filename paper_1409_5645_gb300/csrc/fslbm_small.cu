@@ -113,8 +113,8 @@ __global__ void __launch_bounds__(256, 1) k_steps(Par p, View<P> v, int steps, u
         Geo<R> G;
         R nn, kopen;
         const bool ok = coop_stencil<R, SIG>(p, v.flags, v.phin, x, y, z, in3, (int)i, phic, nn, kopen, G);
+        if (ok) coop_finish<R, SIG, false>(p, v.flags, v.phin, x, y, z, phic, nn, kopen, G);
         if (lane == 0) {
-          if (ok) geometry_finish<R, SIG, false>(p, v.flags, v.phin, x, y, z, phic, nn, &kopen, G);
           v.geo[e] = ok ? G.n[0] : R(0);
           v.geo[cap + e] = ok ? G.n[1] : R(0);
           v.geo[2 * cap + e] = ok ? G.n[2] : R(0);

@@ -777,10 +777,8 @@ __global__ void __launch_bounds__(128, P == P16 ? 10 : P == P64 || SIG || ELV ? 
     Geo<R> G;
     R nn, kopen;
     const bool ok = coop_stencil<R, SIG>(p, v.flags, v.phin, x, y, z, in3, (int)i, phic, nn, kopen, G);
-    if (lane == 0) {
-      if (ok) geometry_finish<R, SIG, ELV>(p, v.flags, v.phin, x, y, z, phic, nn, &kopen, G);
-      put(pos, G);
-    }
+    if (ok) coop_finish<R, SIG, ELV>(p, v.flags, v.phin, x, y, z, phic, nn, kopen, G);
+    if (lane == 0) put(pos, G);
   }
 }
 

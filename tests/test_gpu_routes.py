@@ -1,7 +1,6 @@
 """Which way steps go out, from the profiler's record of launches: many steps of
 a small lattice in one launch only where more than four are asked for and the
-kernels are not wanted in order; graphs only after a handle's first sixteen
-steps by kernels."""
+kernels are not wanted in order; graphs only where they pay."""
 import pytest
 
 from paper_1409_5645_gb300 import cases, fslbm
@@ -51,13 +50,20 @@ def test_many_steps_launch():
         assert _count(r, "k_steps") == 1 and _count(r, bulk) == 1
 
 
-def test_graphs_after_the_first_steps():
+def test_graphs_where_they_pay():
+    """A fresh handle: short calls by kernels, for eight steps at once up to its
+    sixteenth such step, for single ones up to its second; a call of sixteen and
+    more by graphs at once."""
     c = cases.dam_break(nx=96, ny=32, nz=32, col_x=32, col_z=22, tau=0.6, g=2e-4)
     g = fslbm.Lattice.from_case(c, precision="f32", bulk_loads="pairs")
-    r = _record(lambda: g.step(8) or g.sync())
-    assert _count(r, "cudaGraphLaunch") == 0 and _count(r, "k_bulk_pairs") == 8
-    g.step(8)
-    r = _record(lambda: g.step(19) or g.sync())
-    assert _count(r, "cudaGraphLaunch") == 5 and _count(r, "k_bulk_pairs") == 19
-    r = _record(lambda: g.step(19) or g.sync())
-    assert _count(r, "cudaGraphLaunch") == 5 and _count(r, "cudaGraphInstantiate") <= 1
+    # 8: a step by kernels (eight to go), one more, six single graphs; 9: two by kernels, seven single graphs
+    for n, launches in ((8, 6), (9, 7), (24, 3), (8, 1), (8, 1)):
+        r = _record(lambda: g.step(n) or g.sync())
+        assert _count(r, "k_bulk_pairs") == n and _count(r, "cudaGraphLaunch") == launches, n
+    g = fslbm.Lattice.from_case(c, precision="f32", bulk_loads="pairs")
+    for launches in (0, 0, 1, 1):
+        r = _record(lambda: g.step(1) or g.sync())
+        assert _count(r, "cudaGraphLaunch") == launches and _count(r, "k_bulk_pairs") == 1
+    g = fslbm.Lattice.from_case(c, precision="f32", bulk_loads="pairs")
+    r = _record(lambda: g.step(16) or g.sync())
+    assert _count(r, "cudaGraphLaunch") == 2 and _count(r, "k_bulk_pairs") == 16

@@ -1,6 +1,7 @@
-"""quot_near, the quotients of one divisor by one division, rounds as a
-division does (built for the host): divisors of the kernels (1 to 18, a
-normal's length and its L1 norm), dividends of every size they have."""
+"""quot_near, the quotients of one divisor by one division, and over_root, a
+vector over its length, round as a division and a square root do (built for
+the host): divisors of the kernels (1 to 18, a normal's length and its L1
+norm), dividends of every size they have, reciprocals off by an ulp too."""
 import os
 import shutil
 import subprocess
@@ -23,6 +24,19 @@ int main() {
     bad += fsl::quot_near(a, b, 1.0 / b) != a / b;
   }
   bad += fsl::quot_near(0.0, 3.0, 1.0 / 3.0) != 0.0;
+  for (int n = 0; n < 1000000; ++n) {
+    const double scale = std::exp(24.0 * (u() - 0.95));
+    const double v[3] = {(u() - 0.5) * scale, (u() - 0.5) * scale, n % 5 ? (u() - 0.5) * scale : 0.0};
+    const double s = v[0] * v[0] + v[1] * v[1] + v[2] * v[2];
+    double w[3] = {v[0], v[1], v[2]};
+    fsl::over_root<false>(w[0], w[1], w[2], s);
+    for (int a = 0; a < 3; ++a) {
+      bad += w[a] != v[a] / std::sqrt(s);
+      const double y = std::nextafter(1.0 / std::sqrt(s), n % 2 ? 0.0 : 1e300);  // (as rsqrt may be)
+      const double t = s * y, len = fma(fma(-t, t, s), 0.5 * y, t);
+      bad += len != std::sqrt(s) || fsl::quot_near(v[a], len, y) != v[a] / len;
+    }
+  }
   std::printf("%lld\n", bad);
 }
 """
