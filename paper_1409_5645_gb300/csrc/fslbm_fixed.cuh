@@ -116,7 +116,8 @@ __host__ __device__ __forceinline__ double double_of_bits(unsigned long long b) 
 __host__ __device__ __forceinline__ double double_of_fix(long long x) { return (double)x * 0x1p-60; }
 
 // The constants of Par from its rates and forces: |lambda| < 2 holds for every
-// tau > 1/2; the forces must leave the operands in range.
+// tau > 1/2; the forces must leave the operands in range, and u_max^2 must be
+// some units of 2^-60 (a guard near 1e-9 is kept by the FP64 collision).
 inline void fix_constants(Par& p) {
   bool ok = !p.compressible && !p.linear_eq;
   for (int a = 0; a < 3; ++a) {
@@ -129,6 +130,7 @@ inline void fix_constants(Par& p) {
   ok = ok && p.lam_p > -2.0 && p.lam_p < 0.0 && p.lam_m > -2.0 && p.lam_m < 0.0;
   p.fx_lp = ok ? llround(p.lam_p * 0x1p62) : 0;
   p.fx_lm = ok ? llround(p.lam_m * 0x1p62) : 0;
+  ok = ok && !(p.umax2 > 0.0 && p.umax2 < 0x1p-30);
   p.fx_um2 = p.umax2 > 0.0 && p.umax2 < 4.0 ? llround(p.umax2 * 0x1p60) : 0x7fffffffffffffffLL;
   p.fix_ok = ok;
 }
