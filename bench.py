@@ -235,49 +235,52 @@ def hbm_peak():
         return 6800.0, "fallback"
 
 
-def kernel_source_sha():
-    """Hash of the bulk and interface kernels' code (comments and blank lines
-    left out, so that a change of wording does not orphan a profile)."""
+BULK_SOURCE = {"f64": "fslbm_bulk64.cu", "f32": "fslbm_pairs.cu", "f16": "fslbm_pairs.cu"}
+
+
+def kernel_sources(form):
+    """The files that a form's bulk kernel (of the bench's loads) is built from:
+    its own and the device headers that it includes."""
+    csrc = os.path.join(ROOT, "paper_1409_5645_gb300", "csrc")
+    names, todo = [], [BULK_SOURCE[form]]
+    while todo:
+        f = todo.pop()
+        if f in names:
+            continue
+        names.append(f)
+        todo += re.findall(r'#include "(\w+\.cuh)"', open(os.path.join(csrc, f)).read())
+    return [os.path.join(csrc, f) for f in sorted(names)]
+
+
+def kernel_source_sha(form):
+    """Hash of the code of a form's bulk kernel (comments and blank lines left
+    out, so that a change of wording does not orphan a profile)."""
     h = hashlib.sha256()
-    for f in ("fslbm_step.cu", "fslbm_step.cuh", "fslbm_staged.cu", "fslbm_pairs.cu", "fslbm_bulk64.cu",
-              "fslbm_fixed.cuh", "fslbm_slow.cuh", "fslbm_pull.cuh", "fslbm_dev.cuh"):
-        text = open(os.path.join(ROOT, "paper_1409_5645_gb300", "csrc", f)).read()
+    for f in kernel_sources(form):
+        text = open(f).read()
         text = re.sub(r"/\*.*?\*/", "", text, flags=re.S)
         code = [ln.split("//")[0].rstrip() for ln in text.splitlines()]
         h.update("\n".join(ln for ln in code if ln.strip()).encode())
     return h.hexdigest()[:16]
 
 
-def ncu_traffic(form):
-    """Per-launch DRAM bytes of k_bulk from the committed ncu summary, scaled
-    to the full lattice; None if absent or taken on other kernel source."""
-    path = os.path.join(ROOT, "profiles", f"k_bulk_dam_break_{form}.md")
+def profile_number(form, name):
+    """A number of the committed ncu summary of a form's bulk kernel; None if
+    absent or taken on other kernel source."""
     try:
-        text = open(path).read()
+        text = open(os.path.join(ROOT, "profiles", f"k_bulk_dam_break_{form}.md")).read()
     except OSError:
         return None
     sha = re.search(r"kernel_source_sha:\s*([0-9a-f]+)", text)
-    val = re.search(r"traffic_bytes_per_launch_full_size:\s*([0-9.eE+]+)", text)
-    if not sha or not val or sha.group(1) != kernel_source_sha():
+    val = re.search(name + r":\s*([0-9.eE+]+)", text)
+    if not sha or not val or sha.group(1) != kernel_source_sha(form):
         return None
     return float(val.group(1))
 
 
-def fp64_counts_per_cell():
-    """(FP64 operations with FMA = 2, FP64 instructions) per liquid-cell
-    update of the FP64 bulk kernel, from the committed ncu instruction counts;
-    None if absent or taken on other kernel source."""
-    path = os.path.join(ROOT, "profiles", "k_bulk_dam_break_f64.md")
-    try:
-        text = open(path).read()
-    except OSError:
-        return None
-    sha = re.search(r"kernel_source_sha:\s*([0-9a-f]+)", text)
-    fl = re.search(r"fp64_flops_per_liquid_cell:\s*([0-9.eE+]+)", text)
-    ins = re.search(r"fp64_instructions_per_liquid_cell:\s*([0-9.eE+]+)", text)
-    if not sha or not fl or not ins or sha.group(1) != kernel_source_sha():
-        return None
-    return float(fl.group(1)), float(ins.group(1))
+def ncu_traffic(form):
+    """Per-launch DRAM bytes of the bulk kernel, scaled to the full lattice."""
+    return profile_number(form, "traffic_bytes_per_launch_full_size")
 
 
 # ---------------------------------------------------------------------------
@@ -544,7 +547,8 @@ def main():
                                / (ms_max / 1e3) / 1e6, 2),
         "roofline": {"bound": "hbm", "achieved": round(achieved, 1), "peak": peak, "unit": "GB/s",
                      "frac": round(achieved / peak, 4), "traffic": ncu_traffic(forms[0]),
-                     "kernel": {"tma": "k_bulk_tma", "async": "k_bulk_async", "pairs": "k_bulk_pairs"}.get(head["bulk_loads"], "k_bulk"),
+                     "kernel": {"tma": "k_bulk_tma", "async": "k_bulk_async", "pairs": "k_bulk_pairs"}.get(
+                         head["bulk_loads"], "k_bulk_fixed" if forms[0] == "f64" else "k_bulk"),
                      "peak_kind": peak_kind,
                      "alg_bytes_per_launch": alg_bulk, "launch_ms": round(bulk_ms, 5),
                      "step": {"frac": round(step_gbs / peak, 4), "achieved": round(step_gbs, 1),
@@ -577,23 +581,14 @@ def main():
                     "bulk_frac": round(bulk / (r["groups_ms"][0] / 1e3) / 1e9 / peak, 4),
                     "kernel_ms_per_step": [round(x, 5) for x in r["groups_ms"]]}
         if f == "f64":
-            # the FP64 bulk kernel against the measured FP64 arithmetic rate:
-            # its FP64 operations per liquid-cell update from the committed ncu
-            # count (instructions of the same kernel source)
-            from paper_1409_5645_gb300 import fslbm
-            rate = fslbm.fp64_rate()
-            cnt = fp64_counts_per_cell()
-            alu = {"bound": "alu", "peak": round(rate, 3), "unit": "TFLOP/s",
-                   "peak_kind": "measured (dependent FMA chains on every SM)"}
-            if cnt:
-                t = r["groups_ms"][0] / 1e3
-                ach = cnt[0] * r["n_liquid"] / t / 1e12
-                # the FP64 pipe issues one FMA, add or multiply per slot: the
-                # instruction rate against the measured FMA instruction rate
-                ins = cnt[1] * r["n_liquid"] / t / 1e12
-                alu.update(achieved=round(ach, 3), frac=round(ach / rate, 4), flops_per_liquid_cell=cnt[0],
-                           instr_frac=round(ins / (rate / 2.0), 4), instructions_per_liquid_cell=cnt[1])
-            other[f]["bulk_alu"] = alu
+            # (the collision is in 64-bit integers: the kernel is bound by the
+            # issue of their instructions, then by DRAM; bulk_frac above is its
+            # share of the copy bandwidth)
+            other[f]["bulk_bound"] = {"bound": "integer issue",
+                                      "integer_instructions_per_liquid_cell":
+                                          profile_number("f64", "integer_instructions_per_liquid_cell"),
+                                      "fp64_instructions_per_liquid_cell":
+                                          profile_number("f64", "fp64_instructions_per_liquid_cell")}
     # the configuration as written (tau = 0.51, Lambda = 3/16): from its
     # initial state for the steps it runs stably (a non-finite density
     # appears between 3500 and 9000 steps)

@@ -439,8 +439,9 @@ int fslbm_check_grid_barrier(int expire, void *stream);
 /* The current device's FP64 arithmetic rate in TFLOP/s (a fused multiply-add
  * counts two): chains of dependent FMAs on every SM, timed with CUDA events
  * on `stream` (NULL = legacy default), best of three after a warm-up run.
- * The ceiling of the FP64 form, whose stream-collide is bound by arithmetic
- * on GB300.  Synchronises the stream.  An implementation property with no
+ * The ceiling of FP64 arithmetic on GB300: of the adjoint's reverse step, the
+ * interface geometry and the steps of an FP64 differentiation (the FP64 form's
+ * other collisions are in integers).  Synchronises the stream.  An implementation property with no
  * counterpart in the paper. */
 int fslbm_fp64_rate(double *tflops, void *stream);
 
