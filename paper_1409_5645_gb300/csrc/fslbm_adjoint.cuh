@@ -109,10 +109,13 @@ __device__ __forceinline__ A eplus_d(const Par& p, int q, A rho, A ux, A uy, A u
 // In FP64 the pipe's two operations a cycle and SM are the bound: there the
 // terms of a link pair are formed once and the components that are zero leave
 // no operation (8x4x64 film, the liquid instance 34 -> 22 us).  The
-// non-equilibrium parts keep the expressions of the general form: near
-// equilibrium they are differences of nearly equal numbers, and the adjoint of
-// the viscosity is a sum over them (other roundings of theirs moved a film's
-// dJ/dnu by 2e-8).  The float form keeps all its expressions.
+// non-equilibrium parts and the adjoint of u in e^+ keep the expressions of the
+// general form: near equilibrium they are differences of nearly equal numbers,
+// and the adjoint of the viscosity is a sum over them that can cancel to 1e-8 of
+// its terms (other roundings of the first moved a film's dJ/dnu by 2e-8; with
+// the -3/2 u.u parts of all links in one term, 2 % of a 200-step film's time
+// less, 28 of 360 films' moved by 1e-9 to 2e-8 of itself, now 2 by 1.3e-9).
+// The float form keeps all its expressions.
 __device__ __forceinline__ void collide_rev64(const Par& p, const double (&f)[19], const double (&ab)[19],
                                               double (&fb)[19], double (&th)[5]) {
   const double lp = p.lam_p, lm = p.lam_m;
@@ -136,19 +139,20 @@ __device__ __forceinline__ void collide_rev64(const Par& p, const double (&f)[19
     if (cy(q)) jy += double(cy(q)) * f[q];
     if (cz(q)) jz += double(cz(q)) * f[q];
   }
-  const double g0 = p.g[0], g1 = p.g[1], g2 = p.g[2], nl = p.linear_eq ? 0.0 : 1.0;
+  const double g0 = p.g[0], g1 = p.g[1], g2 = p.g[2];
   const double u[3] = {jx + 0.5 * g0, jy + 0.5 * g1, jz + 0.5 * g2};
   const double v[3] = {jx - g0 / lm, jy - g1 / lm, jz - g2 / lm};
-  // rest population; dens: sum of w times the adjoints of e^+ (negated), for rho and the -3/2 w u.u part
+  // rest population; dens: sum of w times the adjoints of e^+ (negated), for rho
   const double np0 = f[0] - eplus_d<double>(p, 0, r, u[0], u[1], u[2]), npb0 = lp * ab[0];
   th[0] += np0 * ab[0];
   fb[0] += ab[0] + npb0;
   double dens = (1.0 / 3.0) * npb0, ub[3] = {0.0, 0.0, 0.0}, vb[3] = {0.0, 0.0, 0.0};
+  deplus_du<double>(p, 0, u[0], u[1], u[2], -npb0, ub);
 #pragma unroll
   for (int q = 1; q < 19; q += 2) {
     const int qb = q + 1;
     const double w = q <= 6 ? 1.0 / 18.0 : 1.0 / 36.0;
-    const double cu = nl * dot(u, q), sp = ab[q] + ab[qb], sm = ab[q] - ab[qb];
+    const double sp = ab[q] + ab[qb], sm = ab[q] - ab[qb];
     const double ep = eplus_d<double>(p, q, r, u[0], u[1], u[2]), em = 3.0 * w * dot(v, q);
     const double np = 0.5 * (f[q] + f[qb]) - ep, nm = 0.5 * (f[q] - f[qb]) - em;
     const double npb = lp * sp, nmb = lm * sm;
@@ -157,12 +161,11 @@ __device__ __forceinline__ void collide_rev64(const Par& p, const double (&f)[19
     fb[q] += ab[q] + 0.5 * (npb + nmb);
     fb[qb] += ab[qb] + 0.5 * (npb - nmb);
     dens += w * npb;
-    add(ub, q, -9.0 * w * cu * npb);
+    deplus_du<double>(p, q, u[0], u[1], u[2], -npb, ub);
     add(vb, q, -3.0 * w * nmb);
   }
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
-    ub[a] += 3.0 * nl * dens * u[a];
     th[2 + a] += 0.5 * ub[a] - quot_near(vb[a], lm, p.inv_lam_m);
     ub[a] += vb[a];
   }
